@@ -149,9 +149,9 @@ fourstep_l2_kernel(FourstepL2Args a) {
         }
         // opaque per item: keeps table addresses and loads inside the loop
         const float2 *twp = a.tw;
-        float2 *bufp = smem;
-        int ltp = lt, cp = c;
-        asm volatile("" : "+l"(twp), "+l"(bufp), "+r"(ltp), "+r"(cp));
+        int ltp = lt, cp = c, zero = 0;
+        asm volatile("" : "+l"(twp), "+r"(ltp), "+r"(cp), "+r"(zero));
+        float2 *bufp = smem + zero;  // still visibly shared memory
         run_passes<L, P, D, SC, 0>(v, ltp, bufp, twp, Interleaved<C>{cp});
         if (it.p1) {
           const int col = c0 + c;  // n1; register m holds k2 = lt + T m

@@ -28,7 +28,7 @@ inline KernelEntry stockham_entry() {
   e.P = P;
   e.TB = TB;
   e.threads = TB * (N / P);
-  e.smem = sizeof(float2) * (size_t)TB * N;
+  e.smem = sizeof(float2) * ((size_t)TB * N + shared_tw_entries<N, SC, TWM>());
   fill_radix<SC>(e);
   e.is_default = DEF;
   e.variant = 0;
@@ -83,7 +83,7 @@ inline KernelEntry tmem2_entry() {
   e.P = P;
   e.TB = 1;
   e.threads = (N / 2) / P;
-  e.smem = tmem2_smem_bytes<N>();
+  e.smem = tmem2_smem_bytes<N, SC, TWM>();
   fill_radix<SC>(e);
   e.is_default = DEF;
   e.twm = TWM;

@@ -80,7 +80,9 @@ struct RaggedUnit {
 constexpr int kRagRoutines = 18;
 constexpr int kRagThreads = 512;
 constexpr int kRagMinLog2 = 4, kRagMaxLog2 = 14;
-constexpr size_t kRagSmem = sizeof(float2) * 16384;  // one unit of 32 points per thread
+constexpr int kRagPoints = 16384;    // one unit of 32 points per thread
+constexpr int kRagTwEntries = 2144;  // twiddle rows of the 16384-point routine 32, 32, 16
+constexpr size_t kRagSmem = sizeof(float2) * (kRagPoints + kRagTwEntries);
 
 struct RagRoutine {
   int N, P, twm, npass, radix[4];
@@ -213,6 +215,14 @@ __device__ __forceinline__ int rag_class(const RaggedArgs &A, float2 *smem, cons
   constexpr int T = N / P;
   constexpr bool PL = pairable<N, P, SC>();
   static_assert(W % T == 0, "rows tile the worker");
+  // The whole-CTA rows read their twiddle rows from shared memory, behind
+  // the row buffer (stockham.cuh); the first exchange publishes the copy.
+  constexpr bool SHARED = T == kRagThreads && shared_tw_entries<N, SC, TWM>() > 0;
+  float2 *tws = smem + kRagPoints;
+  if constexpr (SHARED) {
+    static_assert(TwRows<SC>::total() <= kRagTwEntries, "the rows fit their place");
+    TwRows<SC>::copy(tws, A.tw + A.tw_off[routine], wtid, W);
+  }
   const int g = wtid / T, lt = wtid - g * T;
   float2 a[P];
   {
@@ -233,19 +243,22 @@ __device__ __forceinline__ int rag_class(const RaggedArgs &A, float2 *smem, cons
     const float2 *row0 = nullptr;  // static mode: the next unit's one row
     if (!cl.counter && wtid == 0 && un < cl.limit) row0 = A.in + A.units[un].in0;
     // Opaque per unit: keeps the table and buffer addresses from being
-    // hoisted out of the loop into registers (as in the plain kernel).
+    // hoisted out of the loop into registers (as in the plain kernel; the
+    // buffer through an offset, so that it stays visibly shared memory).
     const float2 *twp = A.tw + A.tw_off[routine];
-    float2 *bufp = smem + (size_t)g * N;
-    int ltp = lt;
-    asm volatile("" : "+l"(twp), "+l"(bufp), "+r"(ltp));
+    int ltp = lt, zero = 0;
+    asm volatile("" : "+l"(twp), "+r"(ltp), "+r"(zero));
+    float2 *bufp = smem + g * N + zero;
     const RagHook hk{&A, un, cl.limit, g, wtid, row0, (unsigned)(sizeof(float2) * N)};
     if constexpr (T == kRagThreads) {
-      run_passes_early<N, P, D, SC, 0, TWM, PL>(a, ltp, bufp, twp, hk, NoTw{}, CtaBarrier{});
+      run_passes_early<N, P, D, SC, 0, TWM, PL, RagHook, NoTw, SHARED>(
+          a, ltp, bufp, SHARED ? tws + zero : twp, hk, NoTw{}, CtaBarrier{});
     } else if constexpr (T >= 64) {
-      run_passes_early<N, P, D, SC, 0, TWM, PL>(a, ltp, bufp, twp, hk, NoTw{},
-                                                NamedBarrier{1 + wid * 4 + g, T});
+      run_passes_early<N, P, D, SC, 0, TWM, PL, RagHook, NoTw, false>(
+          a, ltp, bufp, twp, hk, NoTw{}, NamedBarrier{1 + wid * 4 + g, T});
     } else {
-      run_passes_early<N, P, D, SC, 0, TWM, PL>(a, ltp, bufp, twp, hk, NoTw{}, WarpBarrier{});
+      run_passes_early<N, P, D, SC, 0, TWM, PL, RagHook, NoTw, false>(a, ltp, bufp, twp, hk,
+                                                                      NoTw{}, WarpBarrier{});
     }
     if constexpr (SC::npass == 1) hk();  // no exchange: no hook ran
     // The current and the next unit's descriptors (L1 hits by now).

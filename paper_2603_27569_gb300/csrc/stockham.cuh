@@ -276,19 +276,88 @@ __device__ __forceinline__ void run_passes(float2 (&a)[P], int lt, float2 *buf,
   }
 }
 
+// The table rows a kernel in twiddle mode 1 reads, copied into shared memory
+// once per CTA: pass s keeps its tw_loaded rows back to back (p_s entries
+// each).  Streaming row data evicts the tables from L1 (13 % hit rate
+// measured on a forward + inverse pair at 8192), so a row read through L1
+// mostly waits for L2; from shared memory it costs an LDS.
+template <class SC>
+struct TwRows {
+  template <int r>
+  __host__ __device__ static constexpr int count() {
+    int n = 0;
+    for (int j = 1; j < r; ++j) n += tw_loaded<r>(j);
+    return n;
+  }
+  template <int r>
+  __host__ __device__ static constexpr int row(int j) {  // place of row j among the loaded ones
+    int n = 0;
+    for (int i = 1; i < j; ++i) n += tw_loaded<r>(i);
+    return n;
+  }
+  template <int S = SC::npass>
+  __host__ __device__ static constexpr int offset() {
+    if constexpr (S <= 1) return 0;
+    else return offset<S - 1>() + count<SC::radix[S - 1]>() * SC::stride(S - 1);
+  }
+  __host__ __device__ static constexpr int total() { return offset<>(); }
+
+  // Copies pass S's rows and those of the later passes: thread t of nt.  The
+  // caller's next barrier makes them visible.
+  template <int S = 1>
+  static __device__ __forceinline__ void copy(float2 *dst, const float2 *__restrict__ tw, int t,
+                                              int nt) {
+    if constexpr (S < SC::npass) {
+      constexpr int r = SC::radix[S], p = SC::stride(S);
+#pragma unroll
+      for (int j = 1; j < r; ++j)
+        if (tw_loaded<r>(j))
+          for (int i = 2 * t; i < p; i += 2 * nt)
+            *reinterpret_cast<float4 *>(dst + offset<S>() + row<r>(j) * p + i) = __ldg(
+                reinterpret_cast<const float4 *>(tw + SC::tw_offset(S) + (j - 1) * p + i));
+      copy<S + 1>(dst, tw, t, nt);
+    }
+  }
+};
+
 // Twiddle-table rows of pass S for this thread's butterflies, read ahead:
 // run_passes_early issues these loads before the barrier that precedes the
 // pass's exchange read, so their latency overlaps the barrier wait (the
 // rows do not depend on the exchanged data).  Only the rows the twiddle mode
 // reads are filled; pass_apply derives the rest.
-template <int N, int P, class SC, int S, int TWM, bool PAIRED>
+// SHARED: from the shared-memory copy (TwRows, twiddle mode 1) instead, after
+// the barrier (its latency needs no hiding, and the barrier publishes the
+// first copy).
+template <int N, int P, class SC, int S, int TWM, bool PAIRED, bool SHARED = false>
 struct PassTw {
+  static_assert(!SHARED || TWM == 1, "shared rows are the twiddle mode 1 rows");
   static constexpr int r = SC::radix[S];
   static constexpr int p = SC::stride(S);
   static constexpr int T = N / P;
   static constexpr int Q = P / r;
   float2 w[Q][r];
-  __device__ __forceinline__ void load(int lt, const float2 *__restrict__ tw) {
+  __device__ __forceinline__ void load(int lt, const float2 *tw) {
+    if constexpr (SHARED) {
+      const float2 *rows = tw + TwRows<SC>::template offset<S>();
+#pragma unroll
+      for (int q = 0; q < (PAIRED ? 1 : Q); ++q) {
+        const int k = bfly<T, Q, PAIRED>(lt, q) & (p - 1);
+        const bool ok = FFTGB_OK(k, p, kSiteTwiddle);
+#pragma unroll
+        for (int j = 1; j < r; ++j)
+          if (tw_loaded<r>(j)) {
+            const float2 *e = rows + TwRows<SC>::template row<r>(j) * p + (ok ? k : 0);
+            if constexpr (PAIRED) {
+              const float4 v = *reinterpret_cast<const float4 *>(e);
+              w[0][j] = make_float2(v.x, v.y);
+              w[1][j] = make_float2(v.z, v.w);
+            } else {
+              w[q][j] = *e;
+            }
+          }
+      }
+      return;
+    }
     const float2 *tws = tw + SC::tw_offset(S);
     if constexpr (PAIRED) {
       const int k0 = bfly<T, Q, true>(lt, 0) & (p - 1);
@@ -353,22 +422,25 @@ struct WarpBarrier {
 // run_passes for one row per thread group with the swizzled row layout,
 // reading each pass's twiddle rows ahead of its exchange barrier (PassTw).
 // hk() as in run_passes; br: the group's barrier (the whole CTA by default).
+// SHARED: tw is the shared-memory copy of the rows (TwRows).
 template <int N, int P, int D, class SC, int S, int TWM, bool PAIR_LAST, class HK, class PT,
-          class BR = CtaBarrier>
+          bool SHARED = false, class BR = CtaBarrier>
 __device__ __forceinline__ void run_passes_early(float2 (&a)[P], int lt, float2 *buf,
-                                                 const float2 *__restrict__ tw, const HK &hk,
-                                                 const PT &pre, const BR &br = BR{}) {
+                                                 const float2 *tw, const HK &hk, const PT &pre,
+                                                 const BR &br = BR{}) {
   pass_apply<N, P, D, SC, S, TWM>(a, pre);
   if constexpr (S + 1 < SC::npass) {
     constexpr bool PN = PAIR_LAST && S + 2 == SC::npass;
     if constexpr (S > 0) br.sync();  // every read of the buffer is done
     pass_write<N, P, SC, S>(a, lt, buf, SwizzledRow{});
-    PassTw<N, P, SC, S + 1, TWM, PN> next;
-    next.load(lt, tw);
+    PassTw<N, P, SC, S + 1, TWM, PN, SHARED> next;
+    if constexpr (!SHARED) next.load(lt, tw);
     br.sync();
     if constexpr (S == 0) hk();
     pass_read<N, P, SC, S, SwizzledRow, PN>(a, lt, buf, SwizzledRow{});
-    run_passes_early<N, P, D, SC, S + 1, TWM, PAIR_LAST>(a, lt, buf, tw, hk, next, br);
+    if constexpr (SHARED) next.load(lt, tw);
+    run_passes_early<N, P, D, SC, S + 1, TWM, PAIR_LAST, HK, decltype(next), SHARED>(
+        a, lt, buf, tw, hk, next, br);
   }
 }
 
@@ -424,14 +496,29 @@ __device__ __forceinline__ void load_row(float2 (&a)[P], const float2 *src, int 
 // while this tile's stores drain, instead of being issued after them: the
 // SM's read and write paths to L2 work at the same time.  The buffer is
 // rewritten only after the end-of-tile barrier, so nothing else changes.
+// Twiddle rows in shared memory: for the one-row-per-SM schedules of 16384
+// points and more in twiddle mode 1.  Their persistent CTAs copy the rows
+// once, and with one 16-warp CTA per SM nothing else hides an L1 miss
+// (16384, per 2^25 points: 109 us with generic exchange accesses and rows
+// read through L1, 101 us with neither; 32768 158 / 132 us).  At 8192 and
+// 4096 the read-ahead through L1 stays faster (8192 83.6 us against 91.3 us,
+// 4096 81.5 against 82.7 us): those launches are one CTA per row, so each
+// row would pay for the copy.
+template <int N, class SC, int TWM>
+__host__ __device__ constexpr int shared_tw_entries() {
+  return TWM == 1 && N >= 16384 && SC::npass > 1 ? TwRows<SC>::total() : 0;
+}
+
 template <int N, int P, int TB, int D, class SC, int TWM>
 __global__ void __launch_bounds__(TB *(N / P))
 stockham_kernel(StockhamArgs args) {
+  constexpr bool SHARED = shared_tw_entries<N, SC, TWM>() > 0;
   constexpr bool PAIR_LAST = pairable<N, P, SC>();
   static_assert(SC::product() == N, "radix schedule must multiply to N");
   static_assert(P % SC::max_radix() == 0, "every radix must divide P");
   constexpr int T = N / P;
   extern __shared__ __align__(128) float2 smem[];
+  float2 *tws = smem + TB * N;
   // Launched with programmatic stream serialization: this grid's CTAs may
   // become resident while the previous kernel of the stream is finishing;
   // nothing global is touched before that kernel has completed and its
@@ -463,6 +550,9 @@ stockham_kernel(StockhamArgs args) {
 #pragma unroll
     for (int m = 0; m < P; ++m) a[m] = make_float2(0.f, 0.f);
   }
+  // While the first rows are in flight; the first exchange's barrier
+  // publishes the copy.
+  if constexpr (SHARED) TwRows<SC>::copy(tws, args.tw, threadIdx.x, TB * T);
   for (; tile < ntiles; tile += gridDim.x) {
     const long long next = tile + gridDim.x;
     auto prefetch_next = [&]() {
@@ -484,17 +574,18 @@ stockham_kernel(StockhamArgs args) {
     const bool load_next = next < ntiles && nrow < args.batch;
     // Opaque per tile: keeps the compiler from hoisting the loop-invariant
     // twiddle reads and exchange addresses out of the tile loop into
-    // (occupancy-costly) registers.
+    // (occupancy-costly) registers.  The buffer is hidden behind an opaque
+    // offset, not an opaque pointer: the compiler must still see that it is
+    // shared memory, or every exchange access becomes a generic one (measured
+    // per 2^25 points, opaque pointer / offset: 8192 88.9 / 83.6 us).
     const float2 *twp = args.tw;
-    float2 *bufp = buf;
-    int ltp = lt;
-    asm volatile("" : "+l"(twp), "+l"(bufp), "+r"(ltp));
-    run_passes_early<N, P, D, SC, 0, TWM, PAIR_LAST>(
-        a, ltp, bufp, twp,
-        [&]() {
-          if (first) prefetch_next();
-        },
-        NoTw{});
+    int ltp = lt, zero = 0;
+    asm volatile("" : "+l"(twp), "+r"(ltp), "+r"(zero));
+    auto hook = [&]() {
+      if (first) prefetch_next();
+    };
+    run_passes_early<N, P, D, SC, 0, TWM, PAIR_LAST, decltype(hook), NoTw, SHARED>(
+        a, ltp, buf + zero, SHARED ? tws + zero : twp, hook, NoTw{});
     if (active && FFTGB_OK(row, args.batch, kSiteStoreRow) &&
         (!load_next || FFTGB_OK(nrow, args.batch, kSiteLoadRow))) {
       float2 *dst = args.out + row * N;

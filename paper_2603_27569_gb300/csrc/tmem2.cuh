@@ -62,9 +62,9 @@ __device__ __forceinline__ void st_cs_v8(float2 *p, float2 a, float2 b, float2 c
 
 // Shared memory: the H-point exchange buffer, then the tensor-memory address
 // slot and the mbarrier of the second-half copy.
-template <int N>
+template <int N, class SC, int TWM>
 __host__ __device__ constexpr size_t tmem2_smem_bytes() {
-  return sizeof(float2) * (size_t)(N / 2) + 16;
+  return sizeof(float2) * (size_t)(N / 2 + 2 + shared_tw_entries<N / 2, SC, TWM>());
 }
 
 // cos(k pi / 32), k = 0..16, in FP64 (rounded once to FP32 where used).
@@ -221,13 +221,16 @@ __global__ void __launch_bounds__(N / 2 / P, 1) tmem2_kernel(Tmem2Args args) {
   static_assert(NCOL <= 512, "tensor memory has 512 columns");
   constexpr unsigned kHalf = sizeof(float2) * H, kPiece = kHalf / 32;
   static_assert(kPiece % 16 == 0, "bulk copies move multiples of 16 bytes");
-  extern __shared__ __align__(128) float2 smem[];  // tmem2_smem_bytes<N>()
+  extern __shared__ __align__(128) float2 smem[];  // tmem2_smem_bytes<N, SC, TWM>()
+  constexpr bool SHARED = shared_tw_entries<H, SC, TWM>() > 0;
+  float2 *tws = smem + H + 2;  // the twiddle rows (stockham.cuh)
   uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + H);
   uint64_t *bar = reinterpret_cast<uint64_t *>(smem + H) + 1;
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int lt = threadIdx.x, warp = lt >> 5;
   if (warp == 0) tmem_alloc_warp(tslot, NCOL);
+  if constexpr (SHARED) TwRows<SC>::copy(tws, args.tw, lt, T);  // published by the barrier below
   if (lt == 32) {
     mbar_init(bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -268,9 +271,9 @@ __global__ void __launch_bounds__(N / 2 / P, 1) tmem2_kernel(Tmem2Args args) {
       // addresses and the thread's output indices from being hoisted out of
       // the row loop into registers.
       const float2 *twp = args.tw;
-      float2 *bufp = smem;
-      int ltp = lt;
-      asm volatile("" : "+l"(twp), "+l"(bufp), "+r"(ltp));
+      int ltp = lt, zero = 0;
+      asm volatile("" : "+l"(twp), "+r"(ltp), "+r"(zero));
+      float2 *bufp = smem + zero;
       if (h == 0) {
         ok = __syncthreads_and(mbar_wait(bar, par));  // the second half has landed
         if (!ok) break;
@@ -285,7 +288,8 @@ __global__ void __launch_bounds__(N / 2 / P, 1) tmem2_kernel(Tmem2Args args) {
         tmem2_load_chunk<P, 0>(a, tD);
         __syncthreads();  // every thread has read round 0's last exchange
       }
-      run_passes_early<H, P, D, SC, 0, TWM, PAIR_LAST>(a, ltp, bufp, twp, NoHook{}, NoTw{});
+      run_passes_early<H, P, D, SC, 0, TWM, PAIR_LAST, NoHook, NoTw, SHARED>(
+          a, ltp, bufp, SHARED ? tws + zero : twp, NoHook{}, NoTw{});
       if (h == 0) {
         tmem2_park_chunk<P, 0>(a, tD + REGION);
         tmem_wait_st();
