@@ -421,11 +421,12 @@ fft_status_t exec_rows(fft_plan_impl *pl, const float2 *in, float2 *out, int64_t
     a.tw = pl->d_tw + pl->tw_single;
     a.batch = rows;
     a.scale = pl->scale;
+    a.ahead = pl->resident_ctas;
     const int64_t grid = (rows + pl->k_single->TB - 1) / pl->k_single->TB;
     if (grid > 0x7fffffffLL) return FFT_ERR_INVALID_SIZE;
     void *args[] = {&a};
-    FFTGB_CUDA(cudaLaunchKernel(pl->k_single->fn[pl->direction > 0 ? 1 : 0], dim3((unsigned)grid),
-                                dim3(pl->k_single->threads), args, pl->k_single->smem, st));
+    FFTGB_CUDA(launch_pdl(pl->k_single->fn[pl->direction > 0 ? 1 : 0], dim3((unsigned)grid),
+                          dim3(pl->k_single->threads), pl->k_single->smem, st, args));
     return FFT_OK;
   }
   if (pl->path == FFT_PATH_SINGLE_CTA && pl->k_single->kind == KIND_STAGED) {
@@ -637,12 +638,13 @@ static fft_status_t plan_single(fft_plan_impl *pl, const KernelEntry *k, int cta
   if (s != FFT_OK) return s;
   if (k->kind == KIND_STAGED || k->kind == KIND_TMEM2) ctas_per_sm = 1;  // one per SM by design
   pl->ctas_per_sm = k->kind == KIND_SPLIT ? -1 : ctas_per_sm;
-  // One-tile-per-CTA plain kernels from 4096 points on prefetch one resident
-  // wave ahead (measured back to back: 8192 94.6 -> 89.8 us, 4096 -1.5 %);
-  // the shorter rows are HBM-bound already and measured 3-5 % slower with it.
-  pl->resident_ctas = k->kind == KIND_STOCKHAM && ctas_per_sm == 0 && k->N >= 4096
-                          ? persistent_grid(k, -1)
-                          : 0;
+  // One-tile-per-CTA kernels prefetch one resident wave ahead: plain ones from
+  // 4096 points on (measured back to back: 8192 94.6 -> 89.8 us, 4096 -1.5 %;
+  // the shorter rows are HBM-bound already and measured 3-5 % slower with
+  // it), 16-bit-storage ones from 8192 on (16384 99.3 -> 91.6 us, 8192 66.9 ->
+  // 66.4 us; 4096 and below no faster).
+  const int ahead_from = k->kind == KIND_STOCKHAM ? 4096 : k->kind == KIND_HALFIO ? 8192 : 1 << 30;
+  pl->resident_ctas = ctas_per_sm == 0 && k->N >= ahead_from ? persistent_grid(k, -1) : 0;
   pl->grid_ctas = k->kind == KIND_SPLIT ? k->split * resident_clusters(k)  // persistent clusters
                   : ctas_per_sm != 0   ? persistent_grid(k, ctas_per_sm)
                                        : 0;

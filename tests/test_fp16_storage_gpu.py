@@ -92,3 +92,22 @@ def test_bf16_storage_wrong_dtype_and_size():
     with pytest.raises(ValueError):   # two elements per point
         plan(torch.zeros(4 * 256, dtype=torch.bfloat16, device="cuda"))
     plan.close()
+
+
+@pytest.mark.parametrize("N,batch", [(8192, 700), (16384, 301)])
+def test_fp16_storage_many_waves(N, batch):
+    # more rows than are resident at once, so that most rows were prefetched
+    # by an earlier CTA and the last wave prefetches nothing; sampled rows
+    x = synth.gaussian((batch, N), seed=N + 11)
+    xh = to_half_pairs(x)
+    dev = torch.from_numpy(xh).cuda().view(torch.complex32).reshape(batch, N)
+    plan = fg.Plan(N, batch, fg.FFT_FORWARD, precision=fg.FFT_PREC_FP16_STORAGE)
+    y = plan(dev)
+    torch.cuda.synchronize()
+    plan.close()
+    rows = np.r_[0, 1, batch // 2, batch - 2, batch - 1]
+    xin = xh[rows, :, 0].astype(np.float64) + 1j * xh[rows, :, 1].astype(np.float64)
+    yh = y.view(torch.float16).reshape(batch, N, 2)[torch.from_numpy(rows).cuda()]
+    yh = yh.cpu().numpy().astype(np.float64)
+    err = rel_l2_rows(yh[..., 0] + 1j * yh[..., 1], oracle.fft(xin, nthreads=NTHREADS))
+    assert err.max() <= TOL_FP16_STORAGE
