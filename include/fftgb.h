@@ -365,13 +365,13 @@ fft_status_t fft_filter_grad_h(const void *X, const void *G, void *grad_H, int N
 
 /*
  * Fused spectral filter: the forward FFT, the multiplication by H and the
- * inverse FFT of a row run in ONE kernel with the row in registers (after a
- * Stockham transform each thread already holds the points the next
- * transform's first pass reads), so a row crosses HBM once each way.
+ * inverse FFT of a row run in ONE kernel with the row in registers (the
+ * spectrum stays in the order the forward transform leaves it in, which is
+ * the order the inverse starts from), so a row crosses HBM once each way.
  *
  * fft_filter_plan: plan for `batch` rows of N points, N power of two in
  *   [256, 16384] (FFT_ERR_NOT_SUPPORTED otherwise).  Owns the twiddle tables
- *   and the backward pass's grad_H workspace (one row of sums per 32 rows).
+ *   and the backward pass's grad_H workspace (one row of sums per CTA).
  *   Free with fft_destroy.
  * fft_filter_forward: y = IFFT(FFT(x) * H) (conj_h = 1: * conj(H)), inverse
  *   scaled by 1/N; if X_save is non-NULL it also receives FFT(x) (needed by
@@ -382,11 +382,13 @@ fft_status_t fft_filter_grad_h(const void *X, const void *G, void *grad_H, int N
  *   grad_x = IFFT(FFT(g_y) * conj(H)) = F^H(conj(H) * g_z), g_z = FFT(g_y)/N,
  *   grad_H = sum_rows conj(X_saved) * g_z  (per-block sums over fixed row
  *   sets in row order, then a fixed-order pairwise tree: bitwise
- *   reproducible on a given GPU).  N >= 8192: one kernel (its grad_H partial
- *   sums in tensor memory) and the tree; N <= 4096: three kernels (g_z into
- *   grad_x's buffer, the grad_H reduction over 32-row chunks, then grad_x in
- *   place).  grad_x may not overlap g_y or X_saved
+ *   reproducible on a given GPU).  One kernel (its grad_H partial sums in
+ *   tensor memory) and the tree.  grad_x may not overlap g_y or X_saved
  *   (FFT_ERR_INVALID_VALUE).
+ * fft_filter_forward_packed / fft_filter_backward_packed: the same with the
+ *   saved spectrum in the kernels' own order (a permutation of each row that
+ *   depends on N alone), which costs no reordering on either side.  A
+ *   spectrum saved by one is read by the other only.
  * Device pointers, 16-byte aligned; asynchronous on stream.
  * Paper: Sec. IX-A (FFT fused with matched filtering in one kernel) and
  * Sec. II-D (SAR range compression).
@@ -397,6 +399,11 @@ fft_status_t fft_filter_forward(fft_plan_t plan, const void *x, const void *H, v
 fft_status_t fft_filter_backward(fft_plan_t plan, const void *g_y, const void *H,
                                  const void *X_saved, void *grad_x, void *grad_H,
                                  void *stream);
+fft_status_t fft_filter_forward_packed(fft_plan_t plan, const void *x, const void *H,
+                                       void *y, void *X_packed, int conj_h, void *stream);
+fft_status_t fft_filter_backward_packed(fft_plan_t plan, const void *g_y, const void *H,
+                                        const void *X_packed, void *grad_x, void *grad_H,
+                                        void *stream);
 
 /*
  * fft_filter_step: one training step of the spectral filter under the

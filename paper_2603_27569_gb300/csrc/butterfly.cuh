@@ -265,20 +265,18 @@ __device__ __forceinline__ void cmul_pm(float2 a, float2 b, float2 &plus, float2
 
 // Twiddle mode 1: form the rows that are not read as products of rows
 // already formed, W^{(c +- d) k} = W^{c k} W^{+-d k}, the two signs of one
-// (c, d) together (cmul_pm), from rows 1, 4 (and 2 for r = 4, 16 for
-// r = 32); product depth <= 3.
+// (c, d) together (cmul_pm); product depth <= 3.  derive_from_pow2 starts
+// from the rows whose numbers are powers of two, derive_twiddles from rows 1,
+// 4 (and 2 for r = 4, 16 for r = 32), forming rows 2 and 8 first.
 template <int r>
-__device__ __forceinline__ void derive_twiddles(float2 (&w)[r]) {
+__device__ __forceinline__ void derive_from_pow2(float2 (&w)[r]) {
   if constexpr (r == 4) {
     w[3] = cmul(w[2], w[1]);
   } else if constexpr (r == 8) {
-    w[2] = cmul(w[1], w[1]);
     cmul_pm(w[4], w[1], w[5], w[3]);
     w[6] = cmul(w[4], w[2]);
     w[7] = cmul(w[4], w[3]);
   } else if constexpr (r == 16) {
-    w[2] = cmul(w[1], w[1]);
-    w[8] = cmul(w[4], w[4]);
     cmul_pm(w[4], w[1], w[5], w[3]);
     cmul_pm(w[8], w[1], w[9], w[7]);
     cmul_pm(w[8], w[2], w[10], w[6]);
@@ -287,8 +285,6 @@ __device__ __forceinline__ void derive_twiddles(float2 (&w)[r]) {
     w[14] = cmul(w[12], w[2]);
     w[15] = cmul(w[12], w[3]);
   } else if constexpr (r == 32) {
-    w[2] = cmul(w[1], w[1]);
-    w[8] = cmul(w[4], w[4]);
     cmul_pm(w[16], w[4], w[20], w[12]);
     w[24] = cmul(w[16], w[8]);
     w[28] = cmul(w[16], w[12]);
@@ -307,6 +303,12 @@ __device__ __forceinline__ void derive_twiddles(float2 (&w)[r]) {
   } else {
     static_assert(r == 2, "twiddle mode 1 for radix 2, 4, 8, 16, 32");
   }
+}
+template <int r>
+__device__ __forceinline__ void derive_twiddles(float2 (&w)[r]) {
+  if constexpr (r >= 8) w[2] = cmul(w[1], w[1]);
+  if constexpr (r >= 16) w[8] = cmul(w[4], w[4]);
+  derive_from_pow2<r>(w);
 }
 
 __host__ __device__ constexpr int ilog2(int v) { return v <= 1 ? 0 : 1 + ilog2(v >> 1); }

@@ -21,12 +21,34 @@
 // Buffer: row k2 at k2 LDR; E1 keeps t at t, E2 keeps (t0, k1a) at t0 S + k1a.
 // S = RA + 1 and LDR are odd-stepped so that every 8-byte access of a
 // half-warp touches 16 distinct bank pairs.
+//
+// The twiddle rows sit in shared memory (TwRows of the schedule RB, RA, P,
+// whose pass tables are exactly the two this transform needs): measured for
+// one forward + inverse pair over 2^25 points, rows read through L1 / from
+// shared memory: 16384 190 / 155, 8192 173 / 146, 4096 168 / 131, 1024
+// 143 / 119 us (the streaming rows evict the tables: 13 % L1 hits).
+//
+// Packed order: register m of thread lt is entry ((m / 2) T + lt) 2 + (m & 1)
+// of the row, so a saved spectrum moves in coalesced 16-byte accesses.
 #pragma once
 #include <cuda_runtime.h>
+
+#include <type_traits>
 
 #include "stockham.cuh"
 
 namespace fftgb {
+
+// The packed order as plain numbers, for kernels that only move it.
+struct SpecShape {
+  int P, T, G, K, QB, RA, RB;  // P = 0: natural order
+};
+// Frequency held at entry pos of a packed row.
+__host__ __device__ __forceinline__ int spec_freq(const SpecShape &s, int pos) {
+  const int lt = (pos >> 1) % s.T, m = 2 * (pos / (2 * s.T)) + (pos & 1);
+  const int e = (lt % s.G) * s.QB;
+  return (lt / s.G) * s.K + e % s.K + s.P * (e / s.K) + m / s.RB + s.P * s.RA * (m % s.RB);
+}
 
 template <int N_, int P_, int RA_>
 struct SpecRow {
@@ -49,8 +71,22 @@ struct SpecRow {
   }
   static constexpr int LDR = pitch();
   static constexpr int BUF = P * LDR;  // float2 per row
-  // twiddle tables as a Stockham schedule RB, RA, P lays them out
-  static constexpr int TW_INNER = 0, TW_OUTER = (RA - 1) * RB;
+  // twiddle tables as a Stockham schedule RB, RA, P lays them out: pass 1 is
+  // W_T^{t0 k1a}, the last pass W_N^{t k2}
+  using Tables = std::conditional_t<(RA > 1), Sched<RB, RA, P>, Sched<RB, P>>;
+  using Rows = TwRows<Tables, true>;
+  static constexpr int TW = Rows::total();  // shared-memory entries
+  static __host__ __device__ constexpr SpecShape shape() { return {P, T, G, K, QB, RA, RB}; }
+
+  // The r - 1 twiddles of pass S at entry k, from the shared-memory rows.
+  template <int S, int r, int p>
+  static __device__ __forceinline__ void twiddles(float2 (&w)[r], const float2 *tw, int k) {
+    const float2 *rows = tw + Rows::template offset<S>() + k;
+#pragma unroll
+    for (int j = 1; j < r; ++j)
+      if (Rows::template loaded<r>(j)) w[j] = rows[Rows::template row<r>(j) * p];
+    derive_from_pow2<r>(w);
+  }
 
   // The row's threads meet: a warp, the whole CTA, or a named barrier.
   template <int TB>
@@ -90,11 +126,11 @@ struct SpecRow {
   static __device__ __forceinline__ constexpr int sub_a(int q) { return q * (G / RB) * LDR; }
 
   template <int TB>
-  __device__ __forceinline__ void forward(float2 (&v)[P], const float2 *__restrict__ tw) const {
+  __device__ __forceinline__ void forward(float2 (&v)[P], const float2 *tw) const {
     Dft<P, -1>::run(v);
     {
       float2 w[P];
-      load_twiddles<P, T, 1>(w, tw + TW_OUTER, lt);
+      twiddles<Tables::npass - 1, P, T>(w, tw, lt);
 #pragma unroll
       for (int j = 1; j < P; ++j) v[j] = cmul(v[j], w[j]);
     }
@@ -103,7 +139,7 @@ struct SpecRow {
     row_sync<TB>(b);
     if constexpr (RA > 1) {
       float2 w[RA];
-      load_twiddles<RA, RB, 1>(w, tw + TW_INNER, t0);
+      twiddles<1, RA, RB>(w, tw, t0);
 #pragma unroll
       for (int q = 0; q < QA; ++q)
 #pragma unroll
@@ -133,7 +169,7 @@ struct SpecRow {
   }
 
   template <int TB>
-  __device__ __forceinline__ void inverse(float2 (&v)[P], const float2 *__restrict__ tw) const {
+  __device__ __forceinline__ void inverse(float2 (&v)[P], const float2 *tw) const {
 #pragma unroll
     for (int q = 0; q < QB; ++q) {
       float2 d[RB];
@@ -145,7 +181,7 @@ struct SpecRow {
     }
     if constexpr (RA > 1) {
       float2 w[RA];
-      load_twiddles<RA, RB, 1>(w, tw + TW_INNER, t0);
+      twiddles<1, RA, RB>(w, tw, t0);
       __syncwarp();
 #pragma unroll
       for (int q = 0; q < QA; ++q) {
@@ -168,7 +204,7 @@ struct SpecRow {
     row_sync<TB>(b);
     {
       float2 w[P];
-      load_twiddles<P, T, 1>(w, tw + TW_OUTER, lt);
+      twiddles<Tables::npass - 1, P, T>(w, tw, lt);
 #pragma unroll
       for (int j = 0; j < P; ++j) {
         v[j] = col[j * LDR];

@@ -14,6 +14,7 @@
 
 #include "butterfly.cuh"
 #include "plan.h"
+#include "specrow.cuh"
 
 namespace fftgb {
 
@@ -90,7 +91,7 @@ constexpr int64_t kTreeMaxChunks = 4096;  // 512 blocks x 16 x 8 B = 64 KiB
 
 __global__ void __launch_bounds__(kTreeThreads) grad_h_tree_smem_kernel(const float2 *partial,
                                                                        float2 *out, int N,
-                                                                       int nchunk) {
+                                                                       int nchunk, SpecShape shape) {
   extern __shared__ float2 tree[];  // [nblk][kTreeCols] block sums
   const int k0 = blockIdx.x * kTreeCols;
   const int f = threadIdx.x % kTreeCols, lane = threadIdx.x / kTreeCols;
@@ -120,21 +121,22 @@ __global__ void __launch_bounds__(kTreeThreads) grad_h_tree_smem_kernel(const fl
     }
     __syncthreads();
   }
-  if (lane == 0 && on) out[k0 + f] = tree[f];
+  if (lane == 0 && on) out[shape.P ? spec_freq(shape, k0 + f) : k0 + f] = tree[f];
 }
 
-__global__ void copy_row_kernel(const float2 *src, float2 *dst, int N) {
+__global__ void copy_row_kernel(const float2 *src, float2 *dst, int N, SpecShape shape) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < N) dst[k] = src[k];
+  if (k < N) dst[shape.P ? spec_freq(shape, k) : k] = src[k];
 }
 
 static bool pow2(int64_t v) { return v > 0 && (v & (v - 1)) == 0; }
 
 // grad_H[k] = fixed-order pairwise sum over the nchunk rows of partial
 // ([nchunk][N], overwritten): one launch while the rows fit shared memory,
-// else level by level.
-fft_status_t grad_h_tree(float2 *partial, float2 *grad_H, int N, int64_t nchunk,
-                         cudaStream_t st) {
+// else level by level.  shape: the rows' packed order (specrow.cuh; P = 0:
+// natural); grad_H is in natural order either way.
+fft_status_t grad_h_tree(float2 *partial, float2 *grad_H, int N, int64_t nchunk, cudaStream_t st,
+                         const SpecShape &shape) {
   const int threads = 256;
   const unsigned bx = (unsigned)((N + threads - 1) / threads);
   if (nchunk <= kTreeMaxChunks) {
@@ -145,7 +147,7 @@ fft_status_t grad_h_tree(float2 *partial, float2 *grad_H, int N, int64_t nchunk,
                              (int)smem) != cudaSuccess)
       return FFT_ERR_CUDA;
     grad_h_tree_smem_kernel<<<(unsigned)((N + kTreeCols - 1) / kTreeCols), kTreeThreads, smem, st>>>(
-        partial, grad_H, N, (int)nchunk);
+        partial, grad_H, N, (int)nchunk, shape);
     return cuda_status(cudaGetLastError());
   }
   if (nchunk > 65535 * 2) return FFT_ERR_INVALID_SIZE;
@@ -153,7 +155,7 @@ fft_status_t grad_h_tree(float2 *partial, float2 *grad_H, int N, int64_t nchunk,
     const int64_t groups = (nchunk + 2 * h - 1) / (2 * h);
     grad_h_tree_kernel<<<dim3(bx, (unsigned)groups), threads, 0, st>>>(partial, N, nchunk, h);
   }
-  copy_row_kernel<<<bx, threads, 0, st>>>(partial, grad_H, N);
+  copy_row_kernel<<<bx, threads, 0, st>>>(partial, grad_H, N, shape);
   return cuda_status(cudaGetLastError());
 }
 
@@ -206,7 +208,7 @@ fft_status_t fft_filter_grad_h(const void *X, const void *G, void *grad_H, int N
   float2 *part = (float2 *)work;
   grad_h_partial_kernel<<<dim3(bx, (unsigned)nchunk), threads, 0, st>>>(
       (const float2 *)X, (const float2 *)G, part, N, batch);
-  return grad_h_tree(part, (float2 *)grad_H, N, nchunk, st);
+  return grad_h_tree(part, (float2 *)grad_H, N, nchunk, st, SpecShape{});
 }
 
 }  // extern "C"

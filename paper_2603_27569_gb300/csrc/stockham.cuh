@@ -281,18 +281,23 @@ __device__ __forceinline__ void run_passes(float2 (&a)[P], int lt, float2 *buf,
 // each).  Streaming row data evicts the tables from L1 (13 % hit rate
 // measured on a forward + inverse pair at 8192), so a row read through L1
 // mostly waits for L2; from shared memory it costs an LDS.
-template <class SC>
+// POW2: every row whose number is a power of two instead (rows 2 and 8 too).
+template <class SC, bool POW2 = false>
 struct TwRows {
+  template <int r>
+  __host__ __device__ static constexpr bool loaded(int j) {
+    return POW2 ? (j & (j - 1)) == 0 : tw_loaded<r>(j);
+  }
   template <int r>
   __host__ __device__ static constexpr int count() {
     int n = 0;
-    for (int j = 1; j < r; ++j) n += tw_loaded<r>(j);
+    for (int j = 1; j < r; ++j) n += loaded<r>(j);
     return n;
   }
   template <int r>
   __host__ __device__ static constexpr int row(int j) {  // place of row j among the loaded ones
     int n = 0;
-    for (int i = 1; i < j; ++i) n += tw_loaded<r>(i);
+    for (int i = 1; i < j; ++i) n += loaded<r>(i);
     return n;
   }
   template <int S = SC::npass>
@@ -311,7 +316,7 @@ struct TwRows {
       constexpr int r = SC::radix[S], p = SC::stride(S);
 #pragma unroll
       for (int j = 1; j < r; ++j)
-        if (tw_loaded<r>(j))
+        if (loaded<r>(j))
           for (int i = 2 * t; i < p; i += 2 * nt)
             *reinterpret_cast<float4 *>(dst + offset<S>() + row<r>(j) * p + i) = __ldg(
                 reinterpret_cast<const float4 *>(tw + SC::tw_offset(S) + (j - 1) * p + i));

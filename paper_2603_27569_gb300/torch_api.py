@@ -365,8 +365,8 @@ class _FusedSpectralFilterFn(torch.autograd.Function):
         y = torch.empty_like(xc)
         need_grad = ctx.needs_input_grad[0] or ctx.needs_input_grad[1]
         X = torch.empty_like(xc) if need_grad else None
-        B.fft_filter_forward(plan.handle, xc, Hc, y, X, False,
-                             torch.cuda.current_stream(x.device))
+        B.fft_filter_forward_packed(plan.handle, xc, Hc, y, X, False,
+                                    torch.cuda.current_stream(x.device))
         ctx.save_for_backward(X if X is not None else xc, Hc)
         ctx.shape = x.shape
         return y.view(x.shape)
@@ -379,8 +379,8 @@ class _FusedSpectralFilterFn(torch.autograd.Function):
         plan = _filter_plan(N, batch, X.device)
         gx = torch.empty_like(X)
         gH = torch.empty(N, dtype=torch.complex64, device=X.device)
-        B.fft_filter_backward(plan.handle, gy.contiguous(), H, X, gx, gH,
-                              torch.cuda.current_stream(X.device))
+        B.fft_filter_backward_packed(plan.handle, gy.contiguous(), H, X, gx, gH,
+                                     torch.cuda.current_stream(X.device))
         return (gx.view(ctx.shape) if ctx.needs_input_grad[0] else None,
                 gH if ctx.needs_input_grad[1] else None)
 
