@@ -346,24 +346,36 @@ static fft_status_t launch_tmem2(const KernelEntry *k, int dir, const float2 *in
   return FFT_OK;
 }
 
-fft_status_t launch_column(const KernelEntry *k, int dir, const ColumnArgs &ca,
-                           cudaStream_t st) {
-  const int64_t grid = ca.nmat * (ca.ncols / k->TB);
+fft_status_t launch_column(const KernelEntry *k, int dir, const ColumnArgs &ca, cudaStream_t st,
+                           int64_t grid_cap) {
+  int64_t grid = ca.nmat * (ca.ncols / k->TB);
   if (grid <= 0) return FFT_OK;
   if (grid > 0x7fffffffLL) return FFT_ERR_INVALID_SIZE;
-  ColumnArgs a = ca;
+  ColumnLoopArgs a;  // a column_kernel takes its ColumnArgs part
+  static_cast<ColumnArgs &>(a) = ca;
+  a.ntiles = (unsigned)grid;
+  if (k->loop && grid_cap > 0) grid = std::min(grid, grid_cap);
   void *args[] = {&a};
-  // Programmatic dependent launch up to 2048-point columns (the kernels that
-  // carry the griddepcontrol instructions); the 4096-point column kernels (one
-  // CTA of 128 KiB per SM) measured 1-4 % slower with it.
-  if (k->N <= 2048) {
-    FFTGB_CUDA(launch_pdl(k->fn[dir > 0 ? 1 : 0], dim3((unsigned)grid), dim3(k->threads),
-                          k->smem, st, args));
-  } else {
-    FFTGB_CUDA(cudaLaunchKernel(k->fn[dir > 0 ? 1 : 0], dim3((unsigned)grid), dim3(k->threads),
-                                args, k->smem, st));
-  }
+  FFTGB_CUDA(launch_pdl(k->fn[dir > 0 ? 1 : 0], dim3((unsigned)grid), dim3(k->threads), k->smem,
+                        st, args));
   return FFT_OK;
+}
+
+// The plain column kernel for `cols` columns in all (rows of `ncols`): the
+// wider variant where its tiles divide the rows and fill every SM (1024
+// points, 2^25 in all: 92 us with 16 columns, 103 us with 8; with fewer
+// tiles than SMs the narrower ones keep more of them busy).
+static const KernelEntry *plain_column(int L, int64_t ncols, int64_t cols) {
+  const KernelEntry *wide = default_column(L, 3);
+  if (wide && ncols % wide->TB == 0) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+        cols / wide->TB >= sms)
+      return wide;
+    cudaGetLastError();
+  }
+  return default_column(L, 0);
 }
 
 // Single-launch four-step (fourstep_l2.cuh).  Batches whose work-item count
@@ -470,7 +482,7 @@ fft_status_t exec_rows(fft_plan_impl *pl, const float2 *in, float2 *out, int64_t
     c2.ntot = pl->N;
     c2.scale = pl->scale;
     c2.in_extent = c2.out_extent = rows * pl->N;
-    return launch_column(pl->k_col2, pl->direction, c2, st);
+    return launch_column(pl->k_col2, pl->direction, c2, st, pl->grid_ctas);
   }
   if (pl->path == FFT_PATH_TENSORCORE) return tc_exec(pl, in, out, rows, st);
   return FFT_ERR_INVALID_VALUE;
@@ -572,10 +584,12 @@ static fft_status_t plan_fourstep(fft_plan_impl *pl, int want_n1, int l2_rows) {
     segs.insert(segs.end(), a.begin(), a.end());
   } else {
     pl->k_col1 = default_column(n2, 1);
-    pl->k_col2 = default_column(n1, 0);
+    pl->k_col2 = plain_column(n1, n2, n2 * pl->batch);
     s = ensure_smem_attr(pl->k_col1);
     if (s == FFT_OK) s = ensure_smem_attr(pl->k_col2);
     if (s != FFT_OK) return s;
+    if (pl->k_col2->loop && (pl->grid_ctas = persistent_grid(pl->k_col2, -1)) <= 0)
+      return FFT_ERR_CUDA;
     pl->tw_col1 = off;
     auto a = pass_segments(*pl->k_col1, off);
     segs.insert(segs.end(), a.begin(), a.end());
@@ -723,7 +737,7 @@ static fft_status_t exec_long_columns(fft_plan_impl *pl, const float2 *in, float
     c2.scale = pl->scale;
     c2.in_extent = nm * L * nc;
     c2.out_extent = user_extent;
-    s = launch_column(pl->k_col2, pl->direction, c2, st);
+    s = launch_column(pl->k_col2, pl->direction, c2, st, pl->grid_ctas);
     if (s != FFT_OK) return s;
   }
   return FFT_OK;
@@ -1053,7 +1067,7 @@ fft_status_t fft_exec(fft_plan_t plan, const void *in, void *out, void *stream) 
     c.ntot = 0;  // no four-step twiddle on this path
     c.scale = pl->scale;
     c.in_extent = c.out_extent = extent / (int64_t)sizeof(float2);
-    return launch_column(pl->k_col2, pl->direction, c, (cudaStream_t)stream);
+    return launch_column(pl->k_col2, pl->direction, c, (cudaStream_t)stream, pl->grid_ctas);
   }
   if (pl->batch == 0) return FFT_OK;
   fft_status_t s = check_buffers(in, out, elem_bytes(pl) * pl->N * pl->batch);
@@ -1169,7 +1183,7 @@ fft_status_t fft_plan_columns(fft_plan_t *out, int L, int64_t ncols, int64_t nma
     n2 = std::min(512, 1 << ((lg + 1) / 2));
     n1 = L / n2;
   }
-  const KernelEntry *k = default_column(n1, 0);
+  const KernelEntry *k = plain_column(n1, ncols, (ncols > 0 && nmat > 0) ? ncols * nmat * n2 : 0);
   const KernelEntry *k1 = n2 > 1 ? default_column(n2, 2) : nullptr;
   if (!k || (n2 > 1 && !k1)) return FFT_ERR_NOT_SUPPORTED;
   const int tile = k1 ? std::max(k->TB, k1->TB) : k->TB;
@@ -1222,6 +1236,7 @@ fft_status_t fft_plan_columns(fft_plan_t *out, int L, int64_t ncols, int64_t nma
   }
   if (s == FFT_OK) s = ensure_smem_attr(k);
   if (s == FFT_OK && k1) s = ensure_smem_attr(k1);
+  if (s == FFT_OK && k->loop && (pl->grid_ctas = persistent_grid(k, -1)) <= 0) s = FFT_ERR_CUDA;
   if (s == FFT_OK && k1 && chunk > 0 && ncols > 0) {
     pl->scratch_bytes = (int64_t)sizeof(float2) * L * ncols * chunk;
     if (dev_malloc(&pl->d_scratch, (size_t)pl->scratch_bytes) != cudaSuccess) {

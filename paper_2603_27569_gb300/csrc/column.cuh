@@ -55,6 +55,9 @@ struct ColumnArgs {
   int ntot;              // L * ncols, the size of the four-step twiddle
   float scale;
 };
+struct ColumnLoopArgs : ColumnArgs {
+  unsigned ntiles;  // tiles of the launch
+};
 
 // TWM: 0 no twiddle, 1 the row four-step's per-column twiddle (with a
 // transposed store), 2 the per-sub-matrix twiddle of a long column.
@@ -66,14 +69,10 @@ column_kernel(ColumnArgs args) {
   constexpr int T = L / P;
   constexpr int NT = C * T;
   extern __shared__ __align__(128) float2 smem[];
-  // Programmatic dependent launch (see stockham_kernel) up to 2048-point
-  // columns: phase 2 may become resident while phase 1 finishes, but reads
-  // nothing before it completed.  The 4096-point kernels (one 128 KiB CTA
-  // per SM, many waves) are launched plainly and carry neither instruction.
-  if constexpr (L <= 2048) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  }
+  // Programmatic dependent launch (see stockham_kernel): phase 2 may become
+  // resident while phase 1 finishes, but reads nothing before it completed.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int c = threadIdx.x % C;
   const int lt = threadIdx.x / C;
   const int tiles_per_mat = args.ncols / C;
@@ -140,6 +139,121 @@ column_kernel(ColumnArgs args) {
       const long long off = (long long)final_index<L, P, SC>(lt, m) * args.out_row_stride;
       if (FFTGB_OK(base + off, args.out_extent, kSiteColStore)) dst[off] = cscale(a[m], args.scale);
     }
+  }
+}
+
+// Columns of 1024 to 4096 points, plain (no four-step twiddle, row-major
+// store): the tile fills most of an SM, so one CTA per tile leaves the SM's
+// loads, passes and stores one after the other.  Persistent instead: CTA c
+// takes tiles c, c + G, ...; as it stores output register m it refills the
+// register with the next tile's point m, and the tile's row segments were
+// prefetched into L2 at the start of the tile before.  32 points per thread
+// (128 registers: with 16 the loop's strided addresses spill).  Every twiddle
+// row is read from a shared-memory copy made once per CTA.  Measured over
+// 2^25 points, one CTA per tile with 16 points per thread / this: 1024
+// 109 / 92 us with 16 columns, 103 with 8; 2048 137 / 125; 4096 (one launch)
+// 188 / 180; as phase 2 of the row four-step 2^19 227 / 202, 2^20 257 / 245.
+// Addresses are running pointers: per-point offsets from the strides measured
+// 137 us at 2048.  What bounds it: one 16-warp CTA per SM, and at 2048 and 4096
+// row segments of 64 and 32 bytes.
+template <int L, int P, int D, class SC, int S, class LY>
+__device__ __forceinline__ void run_passes_shared(float2 (&a)[P], int lt, float2 *buf,
+                                                  const float2 *tw, const LY &ly) {
+  constexpr int r = SC::radix[S], p = SC::stride(S), T = L / P, Q = P / r;
+  if constexpr (S > 0) {
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const int k = (lt + q * T) & (p - 1);
+      const bool ok = FFTGB_OK(k, p, kSiteTwiddle);
+      const float2 *rows = tw + SC::tw_offset(S) + (ok ? k : 0);
+#pragma unroll
+      for (int j = 1; j < r; ++j) a[q + j * Q] = cmul_dir<D>(a[q + j * Q], rows[(j - 1) * p]);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    float2 v[r];
+#pragma unroll
+    for (int j = 0; j < r; ++j) v[j] = a[q + j * Q];
+    Dft<r, D>::run(v);
+#pragma unroll
+    for (int j = 0; j < r; ++j) a[q + j * Q] = v[j];
+  }
+  if constexpr (S + 1 < SC::npass) {
+    if constexpr (S > 0) __syncthreads();  // every read of the buffer is done
+    pass_write<L, P, SC, S>(a, lt, buf, ly);
+    __syncthreads();
+    pass_read<L, P, SC, S>(a, lt, buf, ly);
+    run_passes_shared<L, P, D, SC, S + 1, LY>(a, lt, buf, tw, ly);
+  }
+}
+
+template <int L, int P, int C, int D, class SC>
+__global__ void __launch_bounds__(C *(L / P), 65536 / (C * (L / P) * 128))
+column_loop_kernel(ColumnLoopArgs args) {
+  static_assert(SC::product() == L, "radix schedule must multiply to L");
+  static_assert(P % SC::max_radix() == 0, "every radix must divide P");
+  constexpr int T = L / P;
+  constexpr int NT = C * T;
+  extern __shared__ __align__(128) float2 smem[];
+  float2 *tws = smem + L * C;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int c = threadIdx.x % C;
+  const int lt = threadIdx.x / C;
+  // element offset of tile t's first column, in the input or the output (the
+  // launcher keeps tile numbers within 31 bits)
+  const unsigned tiles_per_mat = args.ncols / C, nsub = args.nsub > 1 ? args.nsub : 1;
+  auto base = [&](unsigned t, long long mat_stride, long long sub_stride) {
+    const unsigned tm = t / tiles_per_mat, mat = tm / nsub;
+    return mat * mat_stride + (tm - mat * nsub) * sub_stride + (t - tm * tiles_per_mat) * C;
+  };
+  const unsigned ntiles = args.ntiles;
+  unsigned tile = blockIdx.x;
+  float2 a[P];
+  {
+    const long long in = base(tile, args.in_mat_stride, args.in_sub_stride) + c;
+#pragma unroll
+    for (int m = 0; m < P; ++m) {
+      const long long off = in + (long long)(lt + m * T) * args.in_row_stride;
+      a[m] = FFTGB_OK(off, args.in_extent, kSiteColLoad) ? __ldg(args.in + off) : make_float2(0.f, 0.f);
+    }
+  }
+  for (int i = threadIdx.x; i < SC::tw_total(); i += NT) tws[i] = __ldg(args.tw + i);
+  // (published by the first exchange's barrier)
+  for (; tile < ntiles; tile += gridDim.x) {
+    const unsigned next = tile + gridDim.x;
+    const bool load_next = next < ntiles;
+    const long long in = load_next ? base(next, args.in_mat_stride, args.in_sub_stride) : 0;
+    if (load_next) {
+      for (int i = threadIdx.x; i < L; i += NT)
+        if (FFTGB_OK(in + (long long)i * args.in_row_stride, args.in_extent, kSiteColLoad))
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(args.in + in +
+                                                        (long long)i * args.in_row_stride));
+    }
+    // opaque per tile: nothing of the strides or the buffer is kept in
+    // registers through the passes
+    int zero = 0, ltp = lt, irs = args.in_row_stride, ors = args.out_row_stride;
+    asm volatile("" : "+r"(zero), "+r"(ltp), "+r"(irs), "+r"(ors));
+    run_passes_shared<L, P, D, SC, 0>(a, ltp, smem + zero, tws + zero, Interleaved<C>{c});
+    // register m is output row lt + m T (final_index) and input row lt + m T:
+    // two running pointers
+    const long long out = base(tile, args.out_mat_stride, args.out_sub_stride) + c;
+    const float2 *src = args.in + (in + c + (long long)ltp * irs);
+    float2 *dst = args.out + (out + (long long)ltp * ors);
+    const long long istep = (long long)T * irs, ostep = (long long)T * ors;
+#pragma unroll
+    for (int m = 0; m < P; ++m) {
+      static_assert(final_index<L, P, SC>(0, P - 1) == (P - 1) * T, "outputs are T rows apart");
+      if (FFTGB_OK(dst - args.out, args.out_extent, kSiteColStore)) *dst = cscale(a[m], args.scale);
+      dst += ostep;
+      if (load_next) {
+        a[m] = FFTGB_OK(src - args.in, args.in_extent, kSiteColLoad) ? __ldg(src)
+                                                                     : make_float2(0.f, 0.f);
+        src += istep;
+      }
+    }
+    if (load_next) __syncthreads();  // the next tile rewrites the buffer
   }
 }
 

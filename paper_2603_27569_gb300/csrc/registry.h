@@ -29,11 +29,13 @@ struct KernelEntry {
   int radix[8];   // (split: the schedule of the N/K-point part)
   int tw_total;   // entries of the per-pass twiddle tables
   int is_default; // the built-in choice for this (kind, N, variant)
-  int variant;    // column kernels: 0 plain, 1 twiddle + transposed store;
+  int variant;    // column kernels: 0 plain, 1 twiddle + transposed store, 2 long-column
+                  // phase 1, 3 plain with wider tiles;
                   // 16-bit storage: 0 FP16 pairs, 1 BF16 pairs
   int twm;        // twiddle mode: 0 all from tables, 1 rows 1/4(/16) + products
   int slabs;      // staged kernels: slabs held in the TMA ring (0 otherwise)
   int split;      // cluster kernels: CTAs per row, K (0 otherwise)
+  int loop;       // column kernels: 1 for a persistent grid over the launch's tiles
   const void *fn[2];  // [0] forward (D = -1), [1] inverse (D = +1)
 };
 

@@ -452,7 +452,7 @@ __device__ __forceinline__ void run_passes_early(float2 (&a)[P], int lt, float2 
 // Final-pass output index of register m (after run_passes): the last pass
 // has p = N / r, so butterfly i writes j to i + j N / r.
 template <int N, int P, class SC>
-__device__ __forceinline__ int final_index(int lt, int m) {
+__host__ __device__ __forceinline__ constexpr int final_index(int lt, int m) {
   constexpr int r = SC::radix[SC::npass - 1];
   constexpr int Q = P / r;
   constexpr int T = N / P;

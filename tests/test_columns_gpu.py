@@ -255,3 +255,32 @@ def test_bench_column_workload_sampled(L, flags):
     x = xd[:, cols].cpu().numpy().T
     y = yd[:, cols].cpu().numpy().T
     assert rel_l2_rows(y, oracle.fft(x, nthreads=NTHREADS)).max() <= TOL_FP32
+
+
+# The persistent column kernels (1024 to 4096 points): more tiles than resident
+# CTAs, the last round partial, both tile widths at 1024 (16 columns where they
+# divide the rows and fill the GPU, else 8), rows padded by an odd count.
+@pytest.mark.parametrize("L,nmat,ncols,pad,flags", [
+    (1024, 1, 2464, 0, 0), (1024, 3, 816, 7, 0), (1024, 1, 2456, 3, 0), (1024, 1, 16, 0, 0),
+    (2048, 1, 1312, 0, 0), (2048, 2, 616, 1, 0), (2048, 1, 8, 5, 0),
+    (4096, 1, 620, 0, fg.FFT_FLAG_FORCE_SINGLE_CTA),
+    (4096, 3, 212, 9, fg.FFT_FLAG_FORCE_SINGLE_CTA), (1 << 19, 1, 16, 0, 0)])
+@pytest.mark.parametrize("direction", [fg.FFT_FORWARD, fg.FFT_INVERSE])
+def test_persistent_column_tiles(L, nmat, ncols, pad, flags, direction):
+    buf, x, rs, ms = strided_case(L, nmat, ncols, pad, 5 if nmat > 1 else 0, seed=L + ncols)
+    plan = fg.ColumnPlan(L, ncols, nmat, rs, ms, direction, flags)
+    out, got = run_strided(plan, buf, nmat, L, ncols, rs, ms)
+    again = to_dev(buf)
+    plan(again, again)  # in place
+    plan.close()
+    e = out.itemsize
+    inside = np.array(np.lib.stride_tricks.as_strided(
+        to_host(again), shape=(nmat, L, ncols), strides=(ms * e, rs * e, e)))
+    assert np.array_equal(inside.view(np.uint32), got.view(np.uint32))
+    assert np.isfinite(got.view(np.float32)).all()
+    pick = np.unique(np.r_[0, 7, ncols // 2, ncols - 1] % ncols)
+    want = column_oracle(np.ascontiguousarray(x[:, :, pick]), direction == fg.FFT_INVERSE)
+    assert col_err(np.ascontiguousarray(got[:, :, pick]), want).max() <= TOL_FP32
+    touched = np.zeros(out.shape, bool)
+    np.lib.stride_tricks.as_strided(touched, shape=(nmat, L, ncols), strides=(ms, rs, 1))[:] = True
+    assert np.all(out[~touched] == complex(7.0, -7.0))
