@@ -13,14 +13,21 @@
 // the narrowest C = 4).  In shared memory element (row, c) of the tile sits
 // at row * C + c: with C = 16 a half-warp always touches 16 consecutive
 // columns, so every exchange is free of bank conflicts without a swizzle.
-// Phase 1 stores its result transposed (column-major) through a padded
-// shared tile so that the global store is coalesced as well.
+// Phase 1 stores its result transposed (column-major).  From 128 points on
+// the transpose is free: the last exchange is read with the threads dealt
+// out the other way round (consecutive lanes take consecutive outputs of one
+// column, from a padded tile), so the last pass leaves runs of T outputs per
+// column in a warp and the store is coalesced.  (Measured over 2^25 points
+// against one more trip through a padded tile, two barriers and 16 bytes of
+// shared-memory traffic per point: row four-step 2^16 169 -> 158, 2^17 179 ->
+// 167, 2^18 201 -> 183, 2^20 240 -> 221 us.)  Shorter phase 1s stage.
 //
 // Phase-1 twiddle W_N^{c k} for column c and output k: register m of thread
 // lt holds k = lt + T m (T = L / P), so W_N^{c k} = W_N^{c lt} W_N^{c T m},
-// the product of two exact table entries from grids laid out [lt][c] and
-// [m][c]: a warp's loads read C consecutive columns (whole sectors) instead
-// of gathering one sector per element from a table of all N powers.
+// the product of two exact table entries from grids laid out [c][lt] and
+// [c][m]: a warp reads whole rows of the first and 16-byte pieces of one or
+// two rows of the second instead of gathering one sector per element from a
+// table of all N powers.
 //
 // Columns longer than one CTA holds (L = L1 L2 > 4096) run the same two
 // phases down the column instead of along a row: input row n = n1 + L1 n2,
@@ -41,9 +48,9 @@ struct ColumnArgs {
   const float2 *in;
   float2 *out;
   const float2 *tw;      // per-pass tables of the length-L transform
-  const float2 *tw_a;    // TWM 1: W_Ntot^{c lt} at lt * ncols + c; TWM 2:
+  const float2 *tw_a;    // TWM 1: W_Ntot^{c lt} at c * T + lt; TWM 2:
                          // W_Ntot^{j k} at j * L + k for sub-matrix j; else null
-  const float2 *tw_b;    // TWM 1: W_Ntot^{c T m} at m * ncols + c
+  const float2 *tw_b;    // TWM 1: W_Ntot^{c T m} at c * P + m
   long long nmat;        // number of matrices times nsub
   long long in_mat_stride, out_mat_stride;  // elements between matrices
   long long in_sub_stride, out_sub_stride;  // elements between sub-matrices
@@ -58,6 +65,58 @@ struct ColumnArgs {
 struct ColumnLoopArgs : ColumnArgs {
   unsigned ntiles;  // tiles of the launch
 };
+
+// Row pitch of the tile whose last exchange is read transposed: 16 consecutive
+// lanes read outputs lt of one or more columns at distinct bank pairs.
+template <int C, int T>
+__host__ __device__ constexpr int transposed_pitch() {
+  return C + (T < 16 ? 16 / T : 1);
+}
+// Does a phase 1 of L points read its last exchange transposed (a run of at
+// least 8 outputs, and an exchange to do it in)?
+template <int L, int P, class SC>
+__host__ __device__ constexpr bool merged_transpose() {
+  return SC::npass > 1 && L / P >= 8;
+}
+// Padded tile: element (idx, c) at idx * LD + c.
+template <int LD>
+struct PaddedColumns {
+  static constexpr int width = LD;
+  int c;
+  template <int p, int r>
+  __device__ __forceinline__ int at(int idx) const { return idx * LD + c; }
+};
+// run_passes with the last exchange read by thread (lt2, c2) instead of (lt, c).
+template <int L, int P, int D, class SC, int S, int LD>
+__device__ __forceinline__ void run_passes_transposed(float2 (&a)[P], int lt, int c, int lt2,
+                                                      int c2, float2 *buf,
+                                                      const float2 *__restrict__ tw) {
+  pass_compute<L, P, D, SC, S, 0>(a, lt, tw);
+  if constexpr (S > 0) __syncthreads();  // every read of the buffer is done
+  pass_write<L, P, SC, S>(a, lt, buf, PaddedColumns<LD>{c});
+  __syncthreads();
+  if constexpr (S + 2 == SC::npass) {
+    pass_read<L, P, SC, S>(a, lt2, buf, PaddedColumns<LD>{c2});
+    pass_compute<L, P, D, SC, S + 1, 0>(a, lt2, tw);
+  } else {
+    pass_read<L, P, SC, S>(a, lt, buf, PaddedColumns<LD>{c});
+    run_passes_transposed<L, P, D, SC, S + 1, LD>(a, lt, c, lt2, c2, buf, tw);
+  }
+}
+// Register m (output lt + T m of column col) times W_Ntot^{col (lt + T m)}.
+template <int P, int T, int D>
+__device__ __forceinline__ void phase1_twiddle(float2 (&a)[P], int lt, int col,
+                                               const float2 *__restrict__ tw_a,
+                                               const float2 *__restrict__ tw_b) {
+  const float2 wa = __ldg(tw_a + (long long)col * T + lt);
+  const float4 *wb = reinterpret_cast<const float4 *>(tw_b + (long long)col * P);
+#pragma unroll
+  for (int m = 0; m < P; m += 2) {
+    const float4 w = __ldg(wb + m / 2);
+    a[m] = cmul_dir<D>(a[m], cmul(wa, make_float2(w.x, w.y)));
+    a[m + 1] = cmul_dir<D>(a[m + 1], cmul(wa, make_float2(w.z, w.w)));
+  }
+}
 
 // TWM: 0 no twiddle, 1 the row four-step's per-column twiddle (with a
 // transposed store), 2 the per-sub-matrix twiddle of a long column.
@@ -94,16 +153,23 @@ column_kernel(ColumnArgs args) {
                                                                : make_float2(0.f, 0.f);
     }
   }
+  if constexpr (TWM == 1 && TRANSPOSED && merged_transpose<L, P, SC>()) {
+    const int lt2 = threadIdx.x % T, c2 = threadIdx.x / T;
+    run_passes_transposed<L, P, D, SC, 0, transposed_pitch<C, T>()>(a, lt, c, lt2, c2, smem,
+                                                                    args.tw);
+    phase1_twiddle<P, T, D>(a, lt2, c0 + c2, args.tw_a, args.tw_b);
+    const long long base = mat * args.out_mat_stride + (long long)(c0 + c2) * L + lt2;
+    float2 *dst = args.out + base;
+#pragma unroll
+    for (int m = 0; m < P; ++m)  // final_index(lt2, m) = lt2 + T m
+      if (FFTGB_OK(base + m * T, args.out_extent, kSiteColStore))
+        dst[m * T] = cscale(a[m], args.scale);
+    return;
+  }
   run_passes<L, P, D, SC, 0>(a, lt, smem, args.tw, Interleaved<C>{c});
   // a[m] now holds output index final_index(lt, m) of column c0 + c.
   if constexpr (TWM == 1) {
-    const int col = c0 + c;
-    const float2 wa = __ldg(args.tw_a + (long long)lt * args.ncols + col);
-#pragma unroll
-    for (int m = 0; m < P; ++m) {  // final_index(lt, m) = lt + T m
-      const float2 w = cmul(wa, __ldg(args.tw_b + (long long)m * args.ncols + col));
-      a[m] = cmul_dir<D>(a[m], w);
-    }
+    phase1_twiddle<P, T, D>(a, lt, c0 + c, args.tw_a, args.tw_b);
   } else if constexpr (TWM == 2) {
     // W_L^{sub k}: the CTA reads one contiguous row of L entries, a warp at
     // most two adjacent entries per load (all C columns share k).

@@ -25,7 +25,7 @@
 #pragma once
 #include <stdint.h>
 
-#include "stockham.cuh"
+#include "column.cuh"
 
 namespace fftgb {
 
@@ -34,8 +34,8 @@ struct FourstepL2Args {
   float2 *out;
   float2 *ring;            // S slots of chunk_rows * N points
   const float2 *tw;        // pass tables of the L-point schedule
-  const float2 *tw_a;      // W_N^{c lt} at lt * L + c (phase-1 twiddle, as column.cuh)
-  const float2 *tw_b;      // W_N^{c T m} at m * L + c
+  const float2 *tw_a;      // W_N^{c lt} at c * T + lt (phase-1 twiddle, as column.cuh)
+  const float2 *tw_b;      // W_N^{c T m} at c * P + m
   unsigned *counters;      // [0] items claimed, [1] CTAs finished, then nchunks phase-1
                            // done counts and nchunks phase-2 done counts; all zero
                            // between launches (the last CTA to finish clears them)
@@ -152,27 +152,19 @@ fourstep_l2_kernel(FourstepL2Args a) {
         int ltp = lt, cp = c, zero = 0;
         asm volatile("" : "+l"(twp), "+r"(ltp), "+r"(cp), "+r"(zero));
         float2 *bufp = smem + zero;  // still visibly shared memory
-        run_passes<L, P, D, SC, 0>(v, ltp, bufp, twp, Interleaved<C>{cp});
         if (it.p1) {
-          const int col = c0 + c;  // n1; register m holds k2 = lt + T m
-          const float2 wa = __ldg(a.tw_a + lt * L + col);
+          // A[n1][k2] at slot + n1 * L + k2: the last exchange is read
+          // transposed (column.cuh)
+          int lt2 = threadIdx.x % T, c2 = threadIdx.x / T;
+          asm volatile("" : "+r"(lt2), "+r"(c2));
+          run_passes_transposed<L, P, D, SC, 0, transposed_pitch<C, T>()>(v, ltp, cp, lt2, c2, bufp,
+                                                                          twp);
+          phase1_twiddle<P, T, D>(v, lt2, c0 + c2, a.tw_a, a.tw_b);  // register m: k2 = lt2 + T m
+          float2 *dst = slot + (long long)(c0 + c2) * L + lt2;
 #pragma unroll
-          for (int m = 0; m < P; ++m)
-            v[m] = cmul_dir<D>(v[m], cmul(wa, __ldg(a.tw_b + m * L + col)));
-          // A[n1][k2] at slot + n1 * L + k2, through a tile padded to C + 1 columns
-          constexpr int LD = C + 1;
-          __syncthreads();
-#pragma unroll
-          for (int m = 0; m < P; ++m) smem[final_index<L, P, SC>(lt, m) * LD + c] = v[m];
-          __syncthreads();
-          float2 *dst = slot + (long long)c0 * L;
-#pragma unroll
-          for (int u = 0; u < P; ++u) {
-            const int e = threadIdx.x + u * NT;
-            const int cl = e / L, k = e - cl * L;
-            __stcg(dst + e, smem[k * LD + cl]);
-          }
+          for (int m = 0; m < P; ++m) __stcg(dst + m * T, v[m]);
         } else {
+          run_passes<L, P, D, SC, 0>(v, ltp, bufp, twp, Interleaved<C>{cp});
           // consumed: drop this tile's L row segments (C points = 128 bytes) from L2
           __syncthreads();
           for (int q = threadIdx.x; q < L; q += NT)

@@ -118,7 +118,8 @@ inline KernelEntry column_entry() {
   e.P = P;
   e.TB = C;
   e.threads = C * (L / P);
-  e.smem = sizeof(float2) * (size_t)L * (VAR ? C + 1 : C);
+  e.smem = sizeof(float2) * (size_t)L *
+           (!VAR ? C : merged_transpose<L, P, SC>() ? transposed_pitch<C, L / P>() : C + 1);
   fill_radix<SC>(e);
   e.is_default = DEF;
   e.variant = VAR;
@@ -135,7 +136,7 @@ inline KernelEntry fourstep_l2_entry() {
   e.P = P;
   e.TB = C;
   e.threads = C * (L / P);
-  e.smem = sizeof(float2) * (size_t)L * (C + 1);
+  e.smem = sizeof(float2) * (size_t)L * transposed_pitch<C, L / P>();
   fill_radix<SC>(e);
   e.is_default = 0;
   e.variant = 0;
