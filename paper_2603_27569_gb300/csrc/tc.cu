@@ -257,6 +257,9 @@ tc_kernel(TcArgs a) {
   uint32_t *tslot = reinterpret_cast<uint32_t *>(mbar + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const long long ngroups = (a.batch + C::TB - 1) / C::TB;
+  // Programmatic dependent launch (see stockham_kernel).
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   for (int e = tid; e < 256; e += NT) reinterpret_cast<uint4 *>(Bs)[e] = __ldg(a.bimg + e);
   if (tid == 0) {
@@ -589,7 +592,7 @@ fft_status_t tc_exec(fft_plan_impl *pl, const float2 *in, float2 *out, int64_t r
   const int64_t grid = std::min<int64_t>(groups, st->grid_cap);
   void *args[] = {&a};
   return cuda_status(
-      cudaLaunchKernel(st->fn, dim3((unsigned)grid), dim3(st->threads), args, st->smem, stream));
+      launch_pdl(st->fn, dim3((unsigned)grid), dim3(st->threads), st->smem, stream, args));
 }
 
 void tc_destroy(fft_plan_impl *pl) {
