@@ -19,6 +19,8 @@ _TORCH_NAMES = ("Plan", "get_plan", "fft", "ifft", "fft_host", "SpectralFilter",
 def __getattr__(name):
     # torch-level API, imported on first use so that ``synth`` and the
     # C-ABI names stay importable without paying for ``import torch``.
+    # Kept in the module afterwards: this runs once per name.
     if name in _TORCH_NAMES:
-        return getattr(_importlib.import_module(__name__ + ".torch_api"), name)
+        value = globals()[name] = getattr(_importlib.import_module(__name__ + ".torch_api"), name)
+        return value
     raise AttributeError(name)

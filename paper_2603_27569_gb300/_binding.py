@@ -185,10 +185,11 @@ def _ptr(x) -> int | None:
     """Device/host address of a torch tensor, an int, or None."""
     if x is None:
         return None
+    f = getattr(x, "data_ptr", None)
+    if f is not None:
+        return f()
     if isinstance(x, int):
         return x
-    if hasattr(x, "data_ptr"):
-        return x.data_ptr()
     if hasattr(x, "ctypes"):
         return x.ctypes.data
     raise TypeError(f"cannot take the address of {type(x)}")

@@ -45,6 +45,12 @@ def _check_tensor(x: torch.Tensor, N: int, batch: int, what: str,
         raise ValueError(f"{what} has {x.numel()} elements, plan needs {per_point * N * batch}")
 
 
+# The current stream's handle without building a torch.cuda.Stream object
+# (2 to 3 us per call on the host): torch's own accessor where it has one.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or \
+    (lambda index: torch.cuda.current_stream(index).cuda_stream)
+
+
 class Plan:
     """Owns one fft_plan_t on one CUDA device."""
 
@@ -59,6 +65,7 @@ class Plan:
                 self.handle = B.fft_plan_ex(N, batch, direction, precision, flags)
         self.N, self.batch, self.direction = N, batch, direction
         self.precision, self.flags = precision, flags
+        self._fft_exec = B.lib().fft_exec
 
     def __call__(self, x: torch.Tensor, out: torch.Tensor | None = None, stream=None):
         return self.exec(x, out, stream)
@@ -81,8 +88,13 @@ class Plan:
             out = torch.empty_like(x)
         else:
             _check_tensor(out, self.N, self.batch, "output", self.dtype)
-        st = torch.cuda.current_stream(self.device) if stream is None else stream
-        B.fft_exec(self.handle, x, out, st)
+        if stream is not None:
+            B.fft_exec(self.handle, x, out, stream)
+            return out
+        status = self._fft_exec(self.handle, x.data_ptr(), out.data_ptr(),
+                                _raw_stream(x.get_device()))
+        if status:
+            raise B.FFTError(status, "fft_exec")
         return out
 
     def exec_host(self, x: torch.Tensor, out: torch.Tensor | None = None, stream=None):
@@ -125,8 +137,10 @@ _CACHE_MAX = 64
 
 def get_plan(N: int, batch: int, direction: int, precision: int = 0, flags: int = 0,
              device=None) -> Plan:
-    dev = torch.device("cuda", torch.cuda.current_device()) if device is None \
-        else torch.device(device)
+    if device is None:
+        dev = torch.device("cuda", torch.cuda.current_device())
+    else:
+        dev = device if isinstance(device, torch.device) else torch.device(device)
     key = (dev.index, N, batch, direction, precision, flags)
     with _cache_lock:
         p = _cache.get(key)
@@ -151,7 +165,8 @@ def _raw(x: torch.Tensor, direction: int, precision: int, flags: int, out=None) 
     N = x.shape[-1]
     batch = x.numel() // N if N else 0
     plan = get_plan(N, batch, direction, precision, flags, x.device)
-    return plan.exec(x.contiguous(), out).view(x.shape)
+    y = plan.exec(x.contiguous(), out)
+    return y if y.shape == x.shape else y.view(x.shape)
 
 
 class _FFTFn(torch.autograd.Function):
@@ -225,7 +240,7 @@ class ColumnPlan:
         if out is None:
             out = torch.empty_like(x)
         self._check(out, "output")
-        st = torch.cuda.current_stream(self.device) if stream is None else stream
+        st = _raw_stream(x.get_device()) if stream is None else stream
         B.fft_exec(self.handle, x, out, st)
         return out
 
@@ -337,7 +352,8 @@ _fcache: "collections.OrderedDict[tuple, _FilterPlan]" = collections.OrderedDict
 
 
 def _filter_plan(N: int, batch: int, device) -> _FilterPlan:
-    key = (torch.device(device).index, N, batch)
+    dev = device if isinstance(device, torch.device) else torch.device(device)
+    key = (dev.index, N, batch)
     with _cache_lock:
         p = _fcache.get(key)
         if p is not None:
@@ -365,23 +381,21 @@ class _FusedSpectralFilterFn(torch.autograd.Function):
         y = torch.empty_like(xc)
         need_grad = ctx.needs_input_grad[0] or ctx.needs_input_grad[1]
         X = torch.empty_like(xc) if need_grad else None
-        B.fft_filter_forward_packed(plan.handle, xc, Hc, y, X, False,
-                                    torch.cuda.current_stream(x.device))
+        B.fft_filter_forward_packed(plan.handle, xc, Hc, y, X, False, _raw_stream(x.get_device()))
         ctx.save_for_backward(X if X is not None else xc, Hc)
-        ctx.shape = x.shape
-        return y.view(x.shape)
+        ctx.shape, ctx.plan = x.shape, plan  # the plan outlives its cache entry
+        return y if y.shape == x.shape else y.view(x.shape)
 
     @staticmethod
     def backward(ctx, gy):
         X, H = ctx.saved_tensors
-        N = X.shape[-1]
-        batch = X.numel() // N
-        plan = _filter_plan(N, batch, X.device)
         gx = torch.empty_like(X)
-        gH = torch.empty(N, dtype=torch.complex64, device=X.device)
-        B.fft_filter_backward_packed(plan.handle, gy.contiguous(), H, X, gx, gH,
-                                     torch.cuda.current_stream(X.device))
-        return (gx.view(ctx.shape) if ctx.needs_input_grad[0] else None,
+        gH = torch.empty_like(H)
+        B.fft_filter_backward_packed(ctx.plan.handle, gy.contiguous(), H, X, gx, gH,
+                                     _raw_stream(X.get_device()))
+        if gx.shape != ctx.shape:
+            gx = gx.view(ctx.shape)
+        return (gx if ctx.needs_input_grad[0] else None,
                 gH if ctx.needs_input_grad[1] else None)
 
 
@@ -415,17 +429,18 @@ def spectral_filter_step(x: torch.Tensor, H: torch.Tensor, mask: torch.Tensor,
     batch = x.numel() // N
     xc = x.contiguous()
     Hc = H.detach().contiguous()
-    m = mask.to(torch.float32).contiguous()
+    m = (mask if mask.dtype == torch.float32 else mask.to(torch.float32)).contiguous()
     if m.shape != x.shape:
         raise ValueError("mask must have x's shape")
     plan = _filter_plan(N, batch, x.device)
     y = torch.empty_like(xc) if keep_y else None
     gx = torch.empty_like(xc)
-    gH = torch.empty(N, dtype=torch.complex64, device=x.device)
+    gH = torch.empty_like(Hc)
     loss = torch.empty((), dtype=torch.float32, device=x.device)
-    B.fft_filter_step(plan.handle, xc, Hc, m, y, gx, gH, loss,
-                      torch.cuda.current_stream(x.device))
-    return (y.view(x.shape) if keep_y else None), loss, gx.view(x.shape), gH
+    B.fft_filter_step(plan.handle, xc, Hc, m, y, gx, gH, loss, _raw_stream(x.get_device()))
+    if gx.shape != x.shape:
+        y, gx = (y.view(x.shape) if keep_y else None), gx.view(x.shape)
+    return y, loss, gx, gH
 
 
 class SpectralFilter(torch.nn.Module):
