@@ -28,13 +28,13 @@
 // order (five exchanges per pair, generic accesses, twiddle rows through L1;
 // three kernels for the backward below 8192) / now:
 //            forward     + spectrum   backward     step
-//     256    134 / 93    155 / 135    293 / 144    367 / 207
-//    1024    174 / 102   196 / 137    288 / 146    481 / 231
-//    4096    177 / 131   191 / 141    295 / 171    457 / 290
-//    8192    162 / 138   181 / 152    212 / 184    359 / 308
-//   16384    204 / 156   226 / 169    258 / 219    425 / 350
+//     256    134 / 93    155 / 134    293 / 144    367 / 196
+//    1024    174 / 102   196 / 136    288 / 143    481 / 219
+//    4096    177 / 131   191 / 140    295 / 168    457 / 278
+//    8192    162 / 138   181 / 151    212 / 180    359 / 296
+//   16384    204 / 156   226 / 169    258 / 210    425 / 337
 // (spectrum and backward in packed order; in natural order, for callers of
-// the unpacked entry points, 131..196 and 150..256.)
+// the unpacked entry points, 130..196 and 146..249.)
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -309,27 +309,33 @@ filter_bwd_kernel(FilterArgs a) {
     r.template forward<TB>(v, cta.tw);
 #pragma unroll
     for (int m = 0; m < P; ++m) v[m] = cscale(v[m], a.inv_n);  // g_z
-#pragma unroll
-    for (int c = 0; c < P / C; ++c) {
-      float s[2 * C];
-      float2 x[C];
-      tmem_ld(t_sum + 2 * C * c, s);
+    // The spectrum is read one chunk ahead of the sums it goes into.
+    float2 x[2][C];
+    auto load_x = [&](int c) {
 #pragma unroll
       for (int q = 0; q < C; q += 2) {
         const int m = C * c + q;
+        float2 *to = x[c & 1] + q;
         if constexpr (PACKED) {
           const float4 w = on ? __ldcs(reinterpret_cast<const float4 *>(xs + (m / 2 * T + lt) * 2))
                               : make_float4(0.f, 0.f, 0.f, 0.f);
-          x[q] = lo2(w);
-          x[q + 1] = hi2(w);
+          to[0] = lo2(w);
+          to[1] = hi2(w);
         } else {
-          x[q] = on ? xs[r.freq(m)] : make_float2(0.f, 0.f);
-          x[q + 1] = on ? xs[r.freq(m + 1)] : make_float2(0.f, 0.f);
+          to[0] = on ? xs[r.freq(m)] : make_float2(0.f, 0.f);
+          to[1] = on ? xs[r.freq(m + 1)] : make_float2(0.f, 0.f);
         }
       }
+    };
+    load_x(0);
+#pragma unroll
+    for (int c = 0; c < P / C; ++c) {
+      float s[2 * C];
+      tmem_ld(t_sum + 2 * C * c, s);
+      if (c + 1 < P / C) load_x(c + 1);
       tmem_wait_ld(s);
 #pragma unroll
-      for (int q = 0; q < C; ++q) cta.accumulate(s + 2 * q, x[q], v[C * c + q]);
+      for (int q = 0; q < C; ++q) cta.accumulate(s + 2 * q, x[c & 1][q], v[C * c + q]);
       tmem_st(t_sum + 2 * C * c, s);
     }
     cta.multiply(v, t_h);
@@ -368,6 +374,8 @@ struct FilterStepArgs {
 };
 
 __global__ void pack_h_kernel(const float2 *H, float2 *hp, int N, SpecShape s) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < N) hp[i] = H[spec_freq(s, i)];
 }
@@ -490,20 +498,6 @@ filter_step_kernel(FilterStepArgs a) {
     a.loss_part[blockIdx.x] = t;
   }
   cta.release();
-}
-
-// L = the per-CTA loss sums added in a fixed pairwise order (in FP64).
-__global__ void __launch_bounds__(512) loss_tree_kernel(const float *part, int n, float *loss) {
-  __shared__ double s[512];
-  double v = 0.0;
-  for (int i = threadIdx.x; i < n; i += 512) v += (double)part[i];
-  s[threadIdx.x] = v;
-  __syncthreads();
-  for (int h = 256; h > 0; h >>= 1) {
-    if ((int)threadIdx.x < h) s[threadIdx.x] += s[threadIdx.x + h];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *loss = (float)s[0];
 }
 
 struct FilterKernel {
@@ -733,7 +727,7 @@ static fft_status_t filter_backward(fft_plan_t plan, const void *g_y, const void
   if ((s = cuda_status(launch_pdl(k.fn, dim3((unsigned)f->bwd_grid), dim3(f->v.threads),
                                   f->v.smem, st, args))) != FFT_OK)
     return s;
-  return grad_h_tree(f->d_work, (float2 *)grad_H, N, f->bwd_grid, st, f->v.shape);
+  return grad_h_tree(f->d_work, (float2 *)grad_H, N, f->bwd_grid, st, f->v.shape, LossSum{});
 }
 
 fft_status_t fft_filter_forward(fft_plan_t plan, const void *x, const void *H, void *y,
@@ -792,16 +786,18 @@ fft_status_t fft_filter_step(fft_plan_t plan, const void *x, const void *H, cons
   a.tw = pl->d_tw;
   a.batch = pl->batch;
   a.inv_n = 1.0f / (float)N;
-  pack_h_kernel<<<(N + 255) / 256, 256, 0, st>>>((const float2 *)H, f->d_hp, N, f->v.shape);
-  if ((s = cuda_status(cudaGetLastError())) != FFT_OK) return s;
+  const float2 *h = (const float2 *)H;
+  int n = N;
+  void *pack[] = {&h, &f->d_hp, &n, &f->v.shape};
+  if ((s = cuda_status(launch_pdl((const void *)pack_h_kernel, dim3((N + 255) / 256), dim3(256), 0,
+                                  st, pack))) != FFT_OK)
+    return s;
   void *args[] = {&a};
   if ((s = cuda_status(launch_pdl(f->v.step.fn, dim3((unsigned)f->step_grid),
                                   dim3(f->v.threads), f->v.smem, st, args))) != FFT_OK)
     return s;
-  if ((s = grad_h_tree(f->d_work, (float2 *)grad_H, N, f->step_grid, st, f->v.shape)) != FFT_OK)
-    return s;
-  loss_tree_kernel<<<1, 512, 0, st>>>(f->d_loss_part, f->step_grid, loss);
-  return cuda_status(cudaGetLastError());
+  return grad_h_tree(f->d_work, (float2 *)grad_H, N, f->step_grid, st, f->v.shape,
+                     LossSum{f->d_loss_part, f->step_grid, loss});
 }
 
 }  // extern "C"

@@ -142,10 +142,16 @@ fft_status_t ragged_exec(fft_plan_impl *pl, const float2 *in, float2 *out, cudaS
 void ragged_destroy(fft_plan_impl *pl);
 void ragged_clear_choices();  // forget the ragged autotuner's choices
 // grad_H = fixed-order pairwise sum of the nchunk rows of partial, whose
-// entries are in `shape`'s order (spectral.cu)
+// entries are in `shape`'s order; with part, also *out = the n loss sums added
+// in a fixed order (spectral.cu)
 struct SpecShape;
+struct LossSum {
+  const float *part;
+  int n;
+  float *out;
+};
 fft_status_t grad_h_tree(float2 *partial, float2 *grad_H, int N, int64_t nchunk, cudaStream_t st,
-                         const SpecShape &shape);
+                         const SpecShape &shape, const LossSum &loss);
 
 }  // namespace fftgb
 
