@@ -363,7 +363,7 @@ fft_status_t launch_column(const KernelEntry *k, int dir, const ColumnArgs &ca, 
 
 // The plain column kernel for `cols` columns in all (rows of `ncols`): the
 // wider variant where its tiles divide the rows and fill every SM (1024
-// points, 2^25 in all: 92 us with 16 columns, 103 us with 8; with fewer
+// points, 2^25 in all: 92 us with 16 columns, 99 us with 8; with fewer
 // tiles than SMs the narrower ones keep more of them busy).
 static const KernelEntry *plain_column(int L, int64_t ncols, int64_t cols) {
   const KernelEntry *wide = default_column(L, 3);
@@ -1173,10 +1173,10 @@ fft_status_t fft_plan_columns(fft_plan_t *out, int L, int64_t ncols, int64_t nma
   if (route == FFT_FLAG_FORCE_FOURSTEP && L < 2048) return FFT_ERR_NOT_SUPPORTED;
   // Two launches (L = n1 n2, phase 1 of length n2 = min(512, 2^ceil(log2 L /
   // 2)), phase 2 of length n1 <= 4096) beyond one CTA's column, on request
-  // from L = 2048, and by default at 4096 when ncols fills 16-column tiles:
-  // the 4-column single-launch tile measured 188 us over 2^25 points against
-  // 165 us for the two 64-point launches (at 2048 one launch stays ahead,
-  // 138 us against 165 us).
+  // from L = 2048, and by default at 4096 when ncols fills 16-column tiles
+  // (over 2^25 points the two 64-point launches measure 165 us and the
+  // 4-column single launch 164 us, a tie; at 2048 one launch is ahead, 122 us
+  // against 165 us).
   const bool two = L > 4096 || route == FFT_FLAG_FORCE_FOURSTEP ||
                    (L == 4096 && route == 0 && ncols > 0 && ncols % 16 == 0);
   int n1 = L, n2 = 1;

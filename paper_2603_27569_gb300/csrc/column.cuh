@@ -217,14 +217,21 @@ column_kernel(ColumnArgs args) {
 // (128 registers: with 16 the loop's strided addresses spill).  Every twiddle
 // row is read from a shared-memory copy made once per CTA.  Measured over
 // 2^25 points, one CTA per tile with 16 points per thread / this: 1024
-// 109 / 92 us with 16 columns, 103 with 8; 2048 137 / 125; 4096 (one launch)
-// 188 / 180; as phase 2 of the row four-step 2^19 227 / 202, 2^20 257 / 245.
+// 109 / 92 us with 16 columns, 99 with 8; 2048 137 / 122; 4096 (one launch)
+// 188 / 164; as phase 2 of the row four-step 2^19 227 / 202, 2^20 257 / 242.
 // Addresses are running pointers: per-point offsets from the strides measured
 // 137 us at 2048.  What bounds it: one 16-warp CTA per SM, and at 2048 and 4096
 // row segments of 64 and 32 bytes.
-template <int L, int P, int D, class SC, int S, class LY>
-__device__ __forceinline__ void run_passes_shared(float2 (&a)[P], int lt, float2 *buf,
-                                                  const float2 *tw, const LY &ly) {
+//
+// First exchange (stride 1, radix r): thread lt writes rows lt r + j, so the
+// 16 / C threads whose columns share a half-warp write rows r apart, the same
+// banks.  Row x therefore sits at x ^ ((x / r) mod (16 / C)): the write's row
+// becomes lt r + (j ^ (lt mod 16 / C)), and the read's lt + m T only depends
+// on lt where T is a multiple of 16 r / C (checked), so both stay a per-thread
+// base plus constants.
+template <int L, int P, int C, int D, class SC, int S>
+__device__ __forceinline__ void run_passes_shared(float2 (&a)[P], int lt, int c, float2 *buf,
+                                                  const float2 *tw) {
   constexpr int r = SC::radix[S], p = SC::stride(S), T = L / P, Q = P / r;
   if constexpr (S > 0) {
 #pragma unroll
@@ -247,10 +254,32 @@ __device__ __forceinline__ void run_passes_shared(float2 (&a)[P], int lt, float2
   }
   if constexpr (S + 1 < SC::npass) {
     if constexpr (S > 0) __syncthreads();  // every read of the buffer is done
-    pass_write<L, P, SC, S>(a, lt, buf, ly);
+    constexpr int share = 16 / C;  // rows of one half-warp
+    if constexpr (S == 0 && share > 1) {
+      static_assert(Q == 1 && r % share == 0, "one butterfly per thread, rows in groups");
+      static_assert(T % r == 0, "(lt + m T) / r = lt / r + m T / r");
+      const int x = lt & (share - 1);
+#pragma unroll
+      for (int j = 0; j < r; ++j) {
+        const int row = lt * r + (j ^ x);
+        if (FFTGB_OK(row, L, kSiteXchgWrite)) buf[row * C + c] = a[j];
+      }
+    } else {
+      pass_write<L, P, SC, S>(a, lt, buf, Interleaved<C>{c});
+    }
     __syncthreads();
-    pass_read<L, P, SC, S>(a, lt, buf, ly);
-    run_passes_shared<L, P, D, SC, S + 1, LY>(a, lt, buf, tw, ly);
+    if constexpr (S == 0 && share > 1) {
+#pragma unroll
+      for (int m = 0; m < P; ++m) {
+        // ((lt + m T) / r) mod share, m T / r known at compile time
+        const int row = lt + m * T;
+        const int at = row ^ ((lt / r + m * T / r) & (share - 1));
+        a[m] = FFTGB_OK(at, L, kSiteXchgRead) ? buf[at * C + c] : make_float2(0.f, 0.f);
+      }
+    } else {
+      pass_read<L, P, SC, S>(a, lt, buf, Interleaved<C>{c});
+    }
+    run_passes_shared<L, P, C, D, SC, S + 1>(a, lt, c, buf, tw);
   }
 }
 
@@ -301,7 +330,7 @@ column_loop_kernel(ColumnLoopArgs args) {
     // registers through the passes
     int zero = 0, ltp = lt, irs = args.in_row_stride, ors = args.out_row_stride;
     asm volatile("" : "+r"(zero), "+r"(ltp), "+r"(irs), "+r"(ors));
-    run_passes_shared<L, P, D, SC, 0>(a, ltp, smem + zero, tws + zero, Interleaved<C>{c});
+    run_passes_shared<L, P, C, D, SC, 0>(a, ltp, c, smem + zero, tws + zero);
     // register m is output row lt + m T (final_index) and input row lt + m T:
     // two running pointers
     const long long out = base(tile, args.out_mat_stride, args.out_sub_stride) + c;
