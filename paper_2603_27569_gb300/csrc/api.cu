@@ -598,14 +598,15 @@ static fft_status_t plan_fourstep(fft_plan_impl *pl, int want_n1, int l2_rows) {
     segs.insert(segs.end(), b.begin(), b.end());
   }
   pl->tw_big = off;
-  {  // phase-1 twiddle: W_N^{c lt} [c][lt] and W_N^{c T m} [c][m] (column.cuh)
-    const int P1 = pl->k_l2 ? pl->k_l2->P : pl->k_col1->P, T1 = n2 / P1;
+  {  // phase-1 twiddle: W_N^{c lt} and W_N^{c T m}, [c][..] or [..][c] (column.cuh)
+    const KernelEntry *k1 = pl->k_l2 ? pl->k_l2 : pl->k_col1;
+    const int P1 = k1->P, T1 = n2 / P1;
     // (every table before has an even count: the second grid is read 16 bytes
     // at a time)
     TwSeg ga;
     ga.offset = off;
     ga.kind = 2;
-    ga.p = T1;
+    ga.p = k1->tw_by_column ? T1 : n1;
     ga.r = 0;
     ga.step = 1;
     ga.M = pl->N;
@@ -614,7 +615,7 @@ static fft_status_t plan_fourstep(fft_plan_impl *pl, int want_n1, int l2_rows) {
     segs.push_back(ga);
     TwSeg gb = ga;
     gb.offset = off;
-    gb.p = P1;
+    gb.p = k1->tw_by_column ? P1 : n1;
     gb.step = T1;
     gb.count = (int64_t)P1 * n1;
     pl->tw_big2 = off;

@@ -13,7 +13,7 @@
 // the narrowest C = 4).  In shared memory element (row, c) of the tile sits
 // at row * C + c: with C = 16 a half-warp always touches 16 consecutive
 // columns, so every exchange is free of bank conflicts without a swizzle.
-// Phase 1 stores its result transposed (column-major).  From 128 points on
+// Phase 1 stores its result transposed (column-major).  From 256 points on
 // the transpose is free: the last exchange is read with the threads dealt
 // out the other way round (consecutive lanes take consecutive outputs of one
 // column, from a padded tile), so the last pass leaves runs of T outputs per
@@ -27,7 +27,9 @@
 // the product of two exact table entries from grids laid out [c][lt] and
 // [c][m]: a warp reads whole rows of the first and 16-byte pieces of one or
 // two rows of the second instead of gathering one sector per element from a
-// table of all N powers.
+// table of all N powers.  A staged phase 1, whose lanes hold consecutive
+// columns, has them laid out [lt][c] and [m][c] (N = 4096 as 64 x 64: 159 us,
+// with the other layout 193).
 //
 // Columns longer than one CTA holds (L = L1 L2 > 4096) run the same two
 // phases down the column instead of along a row: input row n = n1 + L1 n2,
@@ -48,9 +50,9 @@ struct ColumnArgs {
   const float2 *in;
   float2 *out;
   const float2 *tw;      // per-pass tables of the length-L transform
-  const float2 *tw_a;    // TWM 1: W_Ntot^{c lt} at c * T + lt; TWM 2:
-                         // W_Ntot^{j k} at j * L + k for sub-matrix j; else null
-  const float2 *tw_b;    // TWM 1: W_Ntot^{c T m} at c * P + m
+  const float2 *tw_a;    // TWM 1: W_Ntot^{c lt} at c * T + lt (staged: lt * ncols + c);
+                         // TWM 2: W_Ntot^{j k} at j * L + k for sub-matrix j; else null
+  const float2 *tw_b;    // TWM 1: W_Ntot^{c T m} at c * P + m (staged: m * ncols + c)
   long long nmat;        // number of matrices times nsub
   long long in_mat_stride, out_mat_stride;  // elements between matrices
   long long in_sub_stride, out_sub_stride;  // elements between sub-matrices
@@ -67,16 +69,18 @@ struct ColumnLoopArgs : ColumnArgs {
 };
 
 // Row pitch of the tile whose last exchange is read transposed: 16 consecutive
-// lanes read outputs lt of one or more columns at distinct bank pairs.
-template <int C, int T>
+// lanes read outputs lt of one column at distinct bank pairs.
+template <int C>
 __host__ __device__ constexpr int transposed_pitch() {
-  return C + (T < 16 ? 16 / T : 1);
+  return C + 1;
 }
-// Does a phase 1 of L points read its last exchange transposed (a run of at
-// least 8 outputs, and an exchange to do it in)?
+// Does a phase 1 of L points read its last exchange transposed?  From 256
+// points on, where a warp's runs are whole lines.  With the 64-byte runs of
+// 128 points it gained 2 % at N = 8192..32768 but lost 5 % at 65536 (512 x
+// 128: 174 / 183 us), and 17 % in the single-launch L2 form (167 / 195 us).
 template <int L, int P, class SC>
 __host__ __device__ constexpr bool merged_transpose() {
-  return SC::npass > 1 && L / P >= 8;
+  return SC::npass > 1 && L / P >= 16;
 }
 // Padded tile: element (idx, c) at idx * LD + c.
 template <int LD>
@@ -118,6 +122,18 @@ __device__ __forceinline__ void phase1_twiddle(float2 (&a)[P], int lt, int col,
   }
 }
 
+// The same where consecutive lanes hold consecutive columns (the staged
+// transpose): grids laid out [lt][c] and [m][c].
+template <int P, int D>
+__device__ __forceinline__ void phase1_twiddle_staged(float2 (&a)[P], int lt, int col, int ncols,
+                                                      const float2 *__restrict__ tw_a,
+                                                      const float2 *__restrict__ tw_b) {
+  const float2 wa = __ldg(tw_a + (long long)lt * ncols + col);
+#pragma unroll
+  for (int m = 0; m < P; ++m)
+    a[m] = cmul_dir<D>(a[m], cmul(wa, __ldg(tw_b + (long long)m * ncols + col)));
+}
+
 // TWM: 0 no twiddle, 1 the row four-step's per-column twiddle (with a
 // transposed store), 2 the per-sub-matrix twiddle of a long column.
 template <int L, int P, int C, int D, class SC, int TWM, bool TRANSPOSED>
@@ -155,7 +171,7 @@ column_kernel(ColumnArgs args) {
   }
   if constexpr (TWM == 1 && TRANSPOSED && merged_transpose<L, P, SC>()) {
     const int lt2 = threadIdx.x % T, c2 = threadIdx.x / T;
-    run_passes_transposed<L, P, D, SC, 0, transposed_pitch<C, T>()>(a, lt, c, lt2, c2, smem,
+    run_passes_transposed<L, P, D, SC, 0, transposed_pitch<C>()>(a, lt, c, lt2, c2, smem,
                                                                     args.tw);
     phase1_twiddle<P, T, D>(a, lt2, c0 + c2, args.tw_a, args.tw_b);
     const long long base = mat * args.out_mat_stride + (long long)(c0 + c2) * L + lt2;
@@ -169,7 +185,7 @@ column_kernel(ColumnArgs args) {
   run_passes<L, P, D, SC, 0>(a, lt, smem, args.tw, Interleaved<C>{c});
   // a[m] now holds output index final_index(lt, m) of column c0 + c.
   if constexpr (TWM == 1) {
-    phase1_twiddle<P, T, D>(a, lt, c0 + c, args.tw_a, args.tw_b);
+    phase1_twiddle_staged<P, D>(a, lt, c0 + c, args.ncols, args.tw_a, args.tw_b);
   } else if constexpr (TWM == 2) {
     // W_L^{sub k}: the CTA reads one contiguous row of L entries, a warp at
     // most two adjacent entries per load (all C columns share k).

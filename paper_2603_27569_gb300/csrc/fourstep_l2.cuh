@@ -35,7 +35,7 @@ struct FourstepL2Args {
   float2 *ring;            // S slots of chunk_rows * N points
   const float2 *tw;        // pass tables of the L-point schedule
   const float2 *tw_a;      // W_N^{c lt} at c * T + lt (phase-1 twiddle, as column.cuh)
-  const float2 *tw_b;      // W_N^{c T m} at c * P + m
+  const float2 *tw_b;      // W_N^{c T m} at c * P + m (staged: lt * L + c and m * L + c)
   unsigned *counters;      // [0] items claimed, [1] CTAs finished, then nchunks phase-1
                            // done counts and nchunks phase-2 done counts; all zero
                            // between launches (the last CTA to finish clears them)
@@ -153,16 +153,32 @@ fourstep_l2_kernel(FourstepL2Args a) {
         asm volatile("" : "+l"(twp), "+r"(ltp), "+r"(cp), "+r"(zero));
         float2 *bufp = smem + zero;  // still visibly shared memory
         if (it.p1) {
-          // A[n1][k2] at slot + n1 * L + k2: the last exchange is read
-          // transposed (column.cuh)
-          int lt2 = threadIdx.x % T, c2 = threadIdx.x / T;
-          asm volatile("" : "+r"(lt2), "+r"(c2));
-          run_passes_transposed<L, P, D, SC, 0, transposed_pitch<C, T>()>(v, ltp, cp, lt2, c2, bufp,
-                                                                          twp);
-          phase1_twiddle<P, T, D>(v, lt2, c0 + c2, a.tw_a, a.tw_b);  // register m: k2 = lt2 + T m
-          float2 *dst = slot + (long long)(c0 + c2) * L + lt2;
+          // A[n1][k2] at slot + n1 * L + k2
+          if constexpr (merged_transpose<L, P, SC>()) {  // the last exchange read transposed (column.cuh)
+            int lt2 = threadIdx.x % T, c2 = threadIdx.x / T;
+            asm volatile("" : "+r"(lt2), "+r"(c2));
+            run_passes_transposed<L, P, D, SC, 0, transposed_pitch<C>()>(v, ltp, cp, lt2, c2,
+                                                                            bufp, twp);
+            phase1_twiddle<P, T, D>(v, lt2, c0 + c2, a.tw_a, a.tw_b);  // register m: k2 = lt2 + T m
+            float2 *dst = slot + (long long)(c0 + c2) * L + lt2;
 #pragma unroll
-          for (int m = 0; m < P; ++m) __stcg(dst + m * T, v[m]);
+            for (int m = 0; m < P; ++m) __stcg(dst + m * T, v[m]);
+          } else {  // through a tile padded to C + 1 columns
+            run_passes<L, P, D, SC, 0>(v, ltp, bufp, twp, Interleaved<C>{cp});
+            phase1_twiddle_staged<P, D>(v, ltp, c0 + cp, L, a.tw_a, a.tw_b);
+            constexpr int LD = C + 1;
+            __syncthreads();
+#pragma unroll
+            for (int m = 0; m < P; ++m) smem[final_index<L, P, SC>(lt, m) * LD + c] = v[m];
+            __syncthreads();
+            float2 *dst = slot + (long long)c0 * L;
+#pragma unroll
+            for (int u = 0; u < P; ++u) {
+              const int e = threadIdx.x + u * NT;
+              const int cl = e / L, k = e - cl * L;
+              __stcg(dst + e, smem[k * LD + cl]);
+            }
+          }
         } else {
           run_passes<L, P, D, SC, 0>(v, ltp, bufp, twp, Interleaved<C>{cp});
           // consumed: drop this tile's L row segments (C points = 128 bytes) from L2

@@ -118,8 +118,8 @@ inline KernelEntry column_entry() {
   e.P = P;
   e.TB = C;
   e.threads = C * (L / P);
-  e.smem = sizeof(float2) * (size_t)L *
-           (!VAR ? C : merged_transpose<L, P, SC>() ? transposed_pitch<C, L / P>() : C + 1);
+  e.smem = sizeof(float2) * (size_t)L * (VAR ? transposed_pitch<C>() : C);  // or C + 1, staged
+  e.tw_by_column = VAR && merged_transpose<L, P, SC>();
   fill_radix<SC>(e);
   e.is_default = DEF;
   e.variant = VAR;
@@ -136,7 +136,8 @@ inline KernelEntry fourstep_l2_entry() {
   e.P = P;
   e.TB = C;
   e.threads = C * (L / P);
-  e.smem = sizeof(float2) * (size_t)L * transposed_pitch<C, L / P>();
+  e.smem = sizeof(float2) * (size_t)L * (C + 1);
+  e.tw_by_column = merged_transpose<L, P, SC>();
   fill_radix<SC>(e);
   e.is_default = 0;
   e.variant = 0;

@@ -175,9 +175,9 @@ fft_status_t setup_device(int dev, DeviceSetup **out) {
     off += pass_table_entries(z.k2);
     // (every table before has an even count: the second grid is read 16 bytes
     // at a time)
-    z.twa = off;  // phase-1 twiddle grid W_N^{c lt}, [c][lt]
+    z.twa = off;  // phase-1 twiddle grid W_N^{c lt}, [c][lt] or [lt][c]
     off += (int64_t)T1 * z.n1;
-    z.twb = off;  // phase-1 twiddle grid W_N^{c T m}, [c][m]
+    z.twb = off;  // phase-1 twiddle grid W_N^{c T m}, [c][m] or [m][c]
     off += (int64_t)z.k1->P * z.n1;
   }
   if (off > kTwEntries) return FFT_ERR_NOT_SUPPORTED;
@@ -189,13 +189,15 @@ fft_status_t setup_device(int dev, DeviceSetup **out) {
     if (fill_pass_tables(z.k1, tw, o) != cudaSuccess) return FFT_ERR_CUDA;
     o = z.tw2;
     if (fill_pass_tables(z.k2, tw, o) != cudaSuccess) return FFT_ERR_CUDA;
-    int64_t T1 = z.n2 / z.k1->P, P1 = z.k1->P, step = 1, M = 1 << e;
+    int64_t T1 = z.n2 / z.k1->P, step = 1, M = 1 << e;
+    int64_t cols_a = z.k1->tw_by_column ? T1 : z.n1;
+    int64_t cols_b = z.k1->tw_by_column ? z.k1->P : z.n1;
     int64_t na = (int64_t)(z.n2 / z.k1->P) * z.n1, nb = (int64_t)z.k1->P * z.n1;
     float2 *dst = tw + z.twa;
-    void *aa[] = {&dst, &T1, &step, &M, &na};
+    void *aa[] = {&dst, &cols_a, &step, &M, &na};
     if (launch_gen((const void *)&gen_grid_twiddles, na, aa) != cudaSuccess) return FFT_ERR_CUDA;
     float2 *dstb = tw + z.twb;
-    void *ab[] = {&dstb, &P1, &T1, &M, &nb};
+    void *ab[] = {&dstb, &cols_b, &T1, &M, &nb};
     if (launch_gen((const void *)&gen_grid_twiddles, nb, ab) != cudaSuccess) return FFT_ERR_CUDA;
   }
   if (cudaDeviceSynchronize() != cudaSuccess) return FFT_ERR_CUDA;

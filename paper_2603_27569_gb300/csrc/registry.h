@@ -35,6 +35,8 @@ struct KernelEntry {
   int twm;        // twiddle mode: 0 all from tables, 1 rows 1/4(/16) + products
   int slabs;      // staged kernels: slabs held in the TMA ring (0 otherwise)
   int split;      // cluster kernels: CTAs per row, K (0 otherwise)
+  int tw_by_column;  // phase 1 (column variant 1, L2 four-step): twiddle grids laid out
+                     // [column][..] (merged transpose), else [..][column]
   int loop;       // column kernels: 1 for a persistent grid over the launch's tiles
   const void *fn[2];  // [0] forward (D = -1), [1] inverse (D = +1)
 };
