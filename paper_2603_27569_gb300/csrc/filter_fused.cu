@@ -30,11 +30,11 @@
 //            forward     + spectrum   backward     step
 //     256    134 / 93    155 / 134    293 / 144    367 / 196
 //    1024    174 / 102   196 / 136    288 / 143    481 / 219
-//    4096    177 / 131   191 / 140    295 / 168    457 / 278
-//    8192    162 / 138   181 / 151    212 / 180    359 / 296
-//   16384    204 / 156   226 / 169    258 / 210    425 / 337
+//    4096    177 / 131   191 / 139    295 / 169    457 / 278
+//    8192    162 / 134   181 / 146    212 / 176    359 / 296
+//   16384    204 / 153   226 / 164    258 / 210    425 / 337
 // (spectrum and backward in packed order; in natural order, for callers of
-// the unpacked entry points, 130..196 and 146..249.)
+// the unpacked entry points, 130..190 and 146..245.)
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -140,20 +140,51 @@ struct FilterCta {
     for (int c = 0; c < P / kChunk<P>; ++c) tmem_st(t + 2 * kChunk<P> * c, z);
     tmem_wait_st();
   }
+  // Place of natural-order entry k in the row buffer: reads and writes by
+  // frequency meet 2-way bank conflicts instead of 8-way.
+  static __device__ __forceinline__ constexpr int at(int k) { return k + 2 * (k >> 5); }
+  static_assert(at(N - 1) < R::BUF, "a natural-order row fits the buffer");
+
   // H (or conj(H)) at this thread's frequencies into the array at t, once.
+  // Rows that fill a CTA get it through the row buffer: read in order, in
+  // flight beside the row's own loads (issued between the two calls).  Gathers
+  // from global memory touch 16 lines per warp load there and wait for each
+  // chunk.  Below, gathers touch fewer lines and are shared by the CTA's rows.
+  // Forward of one row / 400 rows / 2^25 points, us, gathered / staged: 1024
+  // 3.6 / 3.9, 3.9 / 4.4, 102 / 103; 4096 4.9 / 4.6, 11.5 / 9.7, 132 / 131;
+  // 8192 8.4 / 7.7, 22.3 / 19.9, 135 / 134; 16384 15.2 / 13.9, 38.2 / 36.5,
+  // 154 / 153.
+  static constexpr bool STAGE_H = TB == 1;
+  __device__ __forceinline__ void fetch_h(const float2 *H) const {
+    if constexpr (STAGE_H) {
+      const uint32_t to = (uint32_t)__cvta_generic_to_shared(buf);
+#pragma unroll
+      for (int m = 0; m < P; ++m) {
+        const int k = lt + m * T;
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(to + 8 * at(k)), "l"(H + k)
+                     : "memory");
+      }
+    }
+  }
   __device__ __forceinline__ void stash_h(const R &r, const float2 *H, bool conj, uint32_t t) const {
     constexpr int C = kChunk<P>;
+    if constexpr (STAGE_H) {
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      R::template row_sync<TB>(b);
+    }
 #pragma unroll
     for (int c = 0; c < P / C; ++c) {
       float h[2 * C];
 #pragma unroll
       for (int q = 0; q < C; ++q) {
-        const float2 w = __ldg(H + r.freq(C * c + q));
+        const int k = r.freq(C * c + q);
+        const float2 w = STAGE_H ? buf[at(k)] : __ldg(H + k);
         h[2 * q] = w.x;
         h[2 * q + 1] = conj ? -w.y : w.y;
       }
       tmem_st(t + 2 * C * c, h);
     }
+    if constexpr (STAGE_H) R::template row_sync<TB>(b);  // the buffer is the transforms' again
     tmem_wait_st();
   }
   // v *= the array at t
@@ -228,6 +259,7 @@ filter_fwd_kernel(FilterArgs a) {
   const int lt = cta.lt;
   const long long ntiles = (a.batch + TB - 1) / TB;
   long long tile = blockIdx.x;
+  cta.fetch_h(a.H);
   float2 v[P];
   {
     const long long row = tile * TB + cta.b;
@@ -244,14 +276,13 @@ filter_fwd_kernel(FilterArgs a) {
     if (a.x_save) {
       float2 *xs = a.x_save + (active ? row : 0) * N;
       if constexpr (NATURAL) {
-        auto at = [](int k) { return k + 2 * (k >> 5); };  // 2-way conflicts instead of 8
         R::template row_sync<TB>(cta.b);  // every sub-row has been read
 #pragma unroll
-        for (int m = 0; m < P; ++m) cta.buf[at(r.freq(m))] = v[m];
+        for (int m = 0; m < P; ++m) cta.buf[cta.at(r.freq(m))] = v[m];
         R::template row_sync<TB>(cta.b);
 #pragma unroll
         for (int m = 0; m < P; ++m)
-          if (active) __stcs(xs + lt + m * T, cta.buf[at(lt + m * T)]);
+          if (active) __stcs(xs + lt + m * T, cta.buf[cta.at(lt + m * T)]);
         R::template row_sync<TB>(cta.b);
       } else if (active) {
 #pragma unroll
@@ -287,6 +318,7 @@ filter_bwd_kernel(FilterArgs a) {
   const uint32_t t_sum = cta.array(0), t_h = cta.array(1);
   const long long ntiles = (a.batch + TB - 1) / TB;
   long long tile = blockIdx.x;
+  cta.fetch_h(a.H);
   float2 v[P];
   {
     const long long row = tile * TB + cta.b;
