@@ -327,6 +327,18 @@ class _SpectralFilterFn(torch.autograd.Function):
         return grad_x, grad_H
 
 
+def _check_filter(x: torch.Tensor, H: torch.Tensor) -> None:
+    """The kernels read N complex64 points of H beside x's rows and write a
+    grad_H of N: an H of another type, length or device is refused."""
+    N = x.shape[-1]
+    if x.dtype != torch.complex64 or H.dtype != torch.complex64:
+        raise TypeError(f"x and H must be torch.complex64, got {x.dtype} and {H.dtype}")
+    if H.shape[-1:] != (N,) or H.numel() != N:
+        raise ValueError(f"H must have shape ({N},), got {tuple(H.shape)}")
+    if H.device != x.device:
+        raise ValueError(f"H must live on {x.device}, not {H.device}")
+
+
 class _FilterPlan:
     """Owns one fused spectral-filter plan (fft_filter_plan)."""
 
@@ -390,7 +402,7 @@ class _FusedSpectralFilterFn(torch.autograd.Function):
     def backward(ctx, gy):
         X, H = ctx.saved_tensors
         gx = torch.empty_like(X)
-        gH = torch.empty_like(H)
+        gH = X.new_empty(ctx.shape[-1])
         B.fft_filter_backward_packed(ctx.plan.handle, gy.contiguous(), H, X, gx, gH,
                                      _raw_stream(X.get_device()))
         if gx.shape != ctx.shape:
@@ -411,6 +423,7 @@ def spectral_filter(x: torch.Tensor, H: torch.Tensor, fused: bool | None = None)
     fused=True runs forward FFT, multiply and inverse FFT in one kernel per row
     (N = 256..16384); fused=False runs them as separate library kernels;
     None picks the faster for N (fused up to FUSED_MAX_N)."""
+    _check_filter(x, H)
     N = x.shape[-1]
     if fused is None:
         fused = N <= FUSED_MAX_N
@@ -425,17 +438,20 @@ def spectral_filter_step(x: torch.Tensor, H: torch.Tensor, mask: torch.Tensor,
     returns (y or None, L, grad_x, grad_H) from one persistent kernel per call
     (C ABI: fft_filter_step; N = 8192 or 16384, x [..., N] complex64, mask the
     same shape as float32)."""
+    _check_filter(x, H)
     N = x.shape[-1]
     batch = x.numel() // N
     xc = x.contiguous()
     Hc = H.detach().contiguous()
+    if mask.device != x.device:
+        raise ValueError(f"mask must live on {x.device}, not {mask.device}")
     m = (mask if mask.dtype == torch.float32 else mask.to(torch.float32)).contiguous()
     if m.shape != x.shape:
         raise ValueError("mask must have x's shape")
     plan = _filter_plan(N, batch, x.device)
     y = torch.empty_like(xc) if keep_y else None
     gx = torch.empty_like(xc)
-    gH = torch.empty_like(Hc)
+    gH = xc.new_empty(N)
     loss = torch.empty((), dtype=torch.float32, device=x.device)
     B.fft_filter_step(plan.handle, xc, Hc, m, y, gx, gH, loss, _raw_stream(x.get_device()))
     if gx.shape != x.shape:
