@@ -97,7 +97,7 @@ struct FilterCta {
   uint32_t tbase, taddr;
 
   // Before the dependency wait: the tables are constant from the plan's
-  // creation on, and tensor memory is the CTA's own.
+  // creation on.
   __device__ __forceinline__ FilterCta(float2 *smem, const float2 *tables) {
     tid = threadIdx.x;
     warp = tid >> 5;
@@ -105,13 +105,23 @@ struct FilterCta {
     lt = tid - b * T;
     buf = smem + b * R::BUF;
     tw = smem + TB * R::BUF;
-    uint32_t *slot = reinterpret_cast<uint32_t *>(tw + R::TW);
     R::Rows::copy(tw, tables, tid, NT);
-    if (warp == 0) tmem_alloc_warp(slot, NCOL);
+  }
+  // After the wait (tmem.cuh): warp 0 allocates, and the barrier publishes the
+  // address and the tables.  The allocation stands behind the first row's
+  // loads, whose latency covers it, except in the step of several rows per
+  // CTA, where the row held across it cost registers (2^25 points, us, before
+  // / behind the loads: step 1024 221 / 232, 2048 241 / 251, 4096 286 / 277;
+  // backward 256 153 / 140, 4096 175 / 168, 8192 179 / 177).
+  __device__ __forceinline__ uint32_t *slot() const { return reinterpret_cast<uint32_t *>(tw + R::TW); }
+  __device__ __forceinline__ void allocate() const {
+    if (warp == 0) tmem_alloc_warp(slot(), NCOL);
+  }
+  __device__ __forceinline__ void publish() {
     tmem_fence_before();
     __syncthreads();
     tmem_fence_after();
-    tbase = *slot;
+    tbase = *slot();
     taddr = tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(2 * P * (warp >> 2));
   }
   __device__ __forceinline__ uint32_t array(int i) const { return taddr + COLS * i; }
@@ -252,9 +262,8 @@ __global__ void __launch_bounds__(TB *R::T, filter_min_ctas<R, TB>(FK_FWD))
 filter_fwd_kernel(FilterArgs a) {
   constexpr int N = R::N, P = R::P, T = R::T;
   extern __shared__ __align__(128) float2 smem[];
-  const FilterCta<R, TB, 1> cta(smem, a.tw);
+  FilterCta<R, TB, 1> cta(smem, a.tw);
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const R r(cta.buf, cta.lt, cta.b);
   const int lt = cta.lt;
   const long long ntiles = (a.batch + TB - 1) / TB;
@@ -266,6 +275,9 @@ filter_fwd_kernel(FilterArgs a) {
     const bool on = row < a.batch;
     cta.load(v, a.in + (on ? row : 0) * N, lt, on);
   }
+  cta.allocate();
+  cta.publish();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   cta.stash_h(r, a.H, a.conj_h, cta.array(0));
   for (; tile < ntiles; tile += gridDim.x) {
     const long long next = tile + gridDim.x;
@@ -310,12 +322,10 @@ __global__ void __launch_bounds__(TB *R::T, filter_min_ctas<R, TB>(FK_BWD))
 filter_bwd_kernel(FilterArgs a) {
   constexpr int N = R::N, P = R::P, T = R::T, C = kChunk<P>;
   extern __shared__ __align__(128) float2 smem[];
-  const FilterCta<R, TB, 2> cta(smem, a.tw);
+  FilterCta<R, TB, 2> cta(smem, a.tw);
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const R r(cta.buf, cta.lt, cta.b);
   const int lt = cta.lt;
-  const uint32_t t_sum = cta.array(0), t_h = cta.array(1);
   const long long ntiles = (a.batch + TB - 1) / TB;
   long long tile = blockIdx.x;
   cta.fetch_h(a.H);
@@ -326,6 +336,10 @@ filter_bwd_kernel(FilterArgs a) {
     cta.load(v, a.in + (on ? row : 0) * N, lt, on);
   }
   cta.prefetch(a.x_save, tile, a.batch, sizeof(float2));
+  cta.allocate();
+  cta.publish();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const uint32_t t_sum = cta.array(0), t_h = cta.array(1);
   cta.stash_h(r, a.H, true, t_h);
   cta.zero(t_sum);
   for (; tile < ntiles; tile += gridDim.x) {
@@ -418,12 +432,11 @@ filter_step_kernel(FilterStepArgs a) {
   constexpr int N = R::N, P = R::P, T = R::T, C = kChunk<P>;
   constexpr int MK = P == 32 ? 16 : 2;  // registers allow 16 beside 32 points, not beside 16
   extern __shared__ __align__(128) float2 smem[];
-  const FilterCta<R, TB, 2> cta(smem, a.tw);
+  FilterCta<R, TB, 2> cta(smem, a.tw);
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if constexpr (TB > 1) cta.allocate();
   const R r(cta.buf, cta.lt, cta.b);
   const int lt = cta.lt;
-  const uint32_t t_sum = cta.array(0), t_x = cta.array(1);
   const long long ntiles = (a.batch + TB - 1) / TB;
   long long tile = blockIdx.x;
   float2 v[P];
@@ -432,6 +445,10 @@ filter_step_kernel(FilterStepArgs a) {
     const bool on = row < a.batch;
     cta.load(v, a.x + (on ? row : 0) * N, lt, on);
   }
+  if constexpr (TB == 1) cta.allocate();
+  cta.publish();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const uint32_t t_sum = cta.array(0), t_x = cta.array(1);
   cta.zero(t_sum);
   float loss = 0.f;
   for (; tile < ntiles; tile += gridDim.x) {

@@ -257,9 +257,9 @@ tc_kernel(TcArgs a) {
   uint32_t *tslot = reinterpret_cast<uint32_t *>(mbar + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const long long ngroups = (a.batch + C::TB - 1) / C::TB;
-  // Programmatic dependent launch (see stockham_kernel).
+  // Programmatic dependent launch (see stockham_kernel), the dependents
+  // released once this CTA holds its tensor memory (tmem.cuh).
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   for (int e = tid; e < 256; e += NT) reinterpret_cast<uint4 *>(Bs)[e] = __ldg(a.bimg + e);
   if (tid == 0) {
@@ -275,6 +275,7 @@ tc_kernel(TcArgs a) {
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const uint32_t tbase = *tslot;
   const int q4 = warp & 3, g4 = warp >> 2;
   bool ok = true;

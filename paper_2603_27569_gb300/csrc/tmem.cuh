@@ -64,6 +64,14 @@ __device__ __forceinline__ void tmem_wait_st() {
 // Allocation of `ncol` columns (a power of two >= 32) by one whole warp; the
 // address lands in *slot (shared memory).  The permit to allocate is given
 // up at once: a CTA allocates once.
+//
+// The allocation blocks until the SM has the columns free, so its place in a
+// kernel launched with programmatic stream serialization matters: a CTA that
+// held columns while it waited for the kernel before it, on an SM where a CTA
+// of that kernel still wanted its own, would wait forever.  Every kernel here
+// therefore allocates after griddepcontrol.wait, and issues
+// griddepcontrol.launch_dependents only behind the barrier that follows the
+// allocation (one thread's trigger counts for the whole CTA).
 __device__ __forceinline__ void tmem_alloc_warp(uint32_t *slot, uint32_t ncol) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                    (uint32_t)__cvta_generic_to_shared(slot)),

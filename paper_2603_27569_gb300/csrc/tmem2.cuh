@@ -227,7 +227,6 @@ __global__ void __launch_bounds__(N / 2 / P, 1) tmem2_kernel(Tmem2Args args) {
   uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + H);
   uint64_t *bar = reinterpret_cast<uint64_t *>(smem + H) + 1;
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int lt = threadIdx.x, warp = lt >> 5;
   if (warp == 0) tmem_alloc_warp(tslot, NCOL);
   if constexpr (SHARED) TwRows<SC>::copy(tws, args.tw, lt, T);  // published by the barrier below
@@ -238,6 +237,7 @@ __global__ void __launch_bounds__(N / 2 / P, 1) tmem2_kernel(Tmem2Args args) {
   tmem_fence_before();
   __syncthreads();
   tmem_fence_after();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // tensor memory held (tmem.cuh)
   // The second half of row r into the exchange buffer (warp 0; the buffer
   // is free: no thread reads it until the copy's barrier completes).
   auto issue_half = [&](int r) {
