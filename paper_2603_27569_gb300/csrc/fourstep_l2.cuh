@@ -147,11 +147,18 @@ fourstep_l2_kernel(FourstepL2Args a) {
 #pragma unroll
           for (int m = 0; m < P; ++m) v[m] = __ldcg(src + (lt + m * T) * L);
         }
-        // opaque per item: keeps table addresses and loads inside the loop
+        // Opaque per item: keeps table addresses and loads inside the loop, the
+        // buffer through an offset so that it stays visibly shared memory.
+        // Columns of 64 points, two warps per CTA, measured faster with the
+        // pointer itself opaque (N = 4096, 2^25 points, chunks of 8 / 16 rows:
+        // 180 / 198 us, with the offset 191 / 204; 16384 166 and 159, 65536
+        // with chunks of 16 rows 161 and 156, so they take the offset).
         const float2 *twp = a.tw;
+        float2 *bufp = smem;
         int ltp = lt, cp = c, zero = 0;
         asm volatile("" : "+l"(twp), "+r"(ltp), "+r"(cp), "+r"(zero));
-        float2 *bufp = smem + zero;  // still visibly shared memory
+        if constexpr (L < 128) asm volatile("" : "+l"(bufp));
+        else bufp = smem + zero;
         if (it.p1) {
           // A[n1][k2] at slot + n1 * L + k2
           if constexpr (merged_transpose<L, P, SC>()) {  // the last exchange read transposed (column.cuh)
