@@ -124,9 +124,10 @@ fft_status_t cuda_status(cudaError_t e) { return e == cudaSuccess ? FFT_OK : FFT
 
 fft_status_t ensure_smem_attr(const KernelEntry *k) {
   if (k->smem > 48 * 1024) {
-    for (int d = 0; d < 2; ++d)
-      FFTGB_CUDA(cudaFuncSetAttribute(k->fn[d], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)k->smem));
+    for (const void *fn : {k->fn[0], k->fn[1], k->fn_tile[0], k->fn_tile[1]})
+      if (fn)
+        FFTGB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)k->smem));
   }
   return FFT_OK;
 }
@@ -262,8 +263,9 @@ fft_status_t launch_stockham(const KernelEntry *k, int dir, const float2 *in, fl
   if (grid_cap > 0 && grid > grid_cap) grid = grid_cap;
   if (grid > 0x7fffffffLL) return FFT_ERR_INVALID_SIZE;
   void *args[] = {&a};
-  FFTGB_CUDA(launch_pdl(k->fn[dir > 0 ? 1 : 0], dim3((unsigned)grid), dim3(k->threads), k->smem,
-                        st, args));
+  const void *const *fn = grid_cap > 0 ? k->fn : k->fn_tile;
+  FFTGB_CUDA(launch_pdl(fn[dir > 0 ? 1 : 0], dim3((unsigned)grid), dim3(k->threads), k->smem, st,
+                        args));
   return FFT_OK;
 }
 

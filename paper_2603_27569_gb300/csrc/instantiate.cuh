@@ -33,8 +33,11 @@ inline KernelEntry stockham_entry() {
   e.is_default = DEF;
   e.variant = 0;
   e.twm = TWM;
-  e.fn[0] = (const void *)&stockham_kernel<N, P, TB, -1, SC, TWM>;
-  e.fn[1] = (const void *)&stockham_kernel<N, P, TB, +1, SC, TWM>;
+  constexpr bool SHARED = shared_tw_entries<N, SC, TWM>() > 0;
+  e.fn[0] = (const void *)&stockham_kernel<N, P, TB, -1, SC, TWM, SHARED>;
+  e.fn[1] = (const void *)&stockham_kernel<N, P, TB, +1, SC, TWM, SHARED>;
+  e.fn_tile[0] = (const void *)&stockham_kernel<N, P, TB, -1, SC, TWM, false>;
+  e.fn_tile[1] = (const void *)&stockham_kernel<N, P, TB, +1, SC, TWM, false>;
   return e;
 }
 

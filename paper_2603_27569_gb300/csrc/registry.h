@@ -39,6 +39,7 @@ struct KernelEntry {
                      // [column][..] (merged transpose), else [..][column]
   int loop;       // column kernels: 1 for a persistent grid over the launch's tiles
   const void *fn[2];  // [0] forward (D = -1), [1] inverse (D = +1)
+  const void *fn_tile[2];  // plain kernels: the same for a plan of one CTA per tile
 };
 
 void register_kernel(const KernelEntry &e);

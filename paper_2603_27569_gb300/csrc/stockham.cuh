@@ -508,16 +508,18 @@ __device__ __forceinline__ void load_row(float2 (&a)[P], const float2 *src, int 
 // read through L1, 101 us with neither; 32768 158 / 132 us).  At 8192 and
 // 4096 the read-ahead through L1 stays faster (8192 83.6 us against 91.3 us,
 // 4096 81.5 against 82.7 us): those launches are one CTA per row, so each
-// row would pay for the copy.
+// row would pay for the copy.  So does a 16384-point plan of one CTA per row,
+// which reads through L1 too (KernelEntry::fn_tile; copied / through L1: 16
+// points per thread 165.7 / 147.3 us, 32 points 116.4 / 115.5).
 template <int N, class SC, int TWM>
 __host__ __device__ constexpr int shared_tw_entries() {
   return TWM == 1 && N >= 16384 && SC::npass > 1 ? TwRows<SC>::total() : 0;
 }
 
-template <int N, int P, int TB, int D, class SC, int TWM>
+// SHARED: see shared_tw_entries.
+template <int N, int P, int TB, int D, class SC, int TWM, bool SHARED>
 __global__ void __launch_bounds__(TB *(N / P))
 stockham_kernel(StockhamArgs args) {
-  constexpr bool SHARED = shared_tw_entries<N, SC, TWM>() > 0;
   constexpr bool PAIR_LAST = pairable<N, P, SC>();
   static_assert(SC::product() == N, "radix schedule must multiply to N");
   static_assert(P % SC::max_radix() == 0, "every radix must divide P");
