@@ -382,8 +382,9 @@ fft_status_t fft_filter_grad_h(const void *X, const void *G, void *grad_H, int N
  *   grad_x = IFFT(FFT(g_y) * conj(H)) = F^H(conj(H) * g_z), g_z = FFT(g_y)/N,
  *   grad_H = sum_rows conj(X_saved) * g_z  (per-block sums over fixed row
  *   sets in row order, then a fixed-order pairwise tree: bitwise
- *   reproducible on a given GPU).  One kernel (its grad_H partial sums in
- *   tensor memory) and the tree.  grad_x may not overlap g_y or X_saved
+ *   reproducible on a given GPU; below 8192 points a set has at most 32 rows
+ *   at any batch, larger batches run as several launches).  One kernel (its
+ *   grad_H partial sums in tensor memory) and the tree.  grad_x may not overlap g_y or X_saved
  *   (FFT_ERR_INVALID_VALUE).
  * fft_filter_forward_packed / fft_filter_backward_packed: the same with the
  *   saved spectrum in the kernels' own order (a permutation of each row that

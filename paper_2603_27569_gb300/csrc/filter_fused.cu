@@ -599,7 +599,7 @@ static bool filter_variant(int N, FilterVariant *v) {
 
 struct FilterState {
   FilterVariant v;
-  float2 *d_work = nullptr;      // per-CTA grad_H sums, one row per CTA
+  float2 *d_work = nullptr;      // grad_H sums, one row per CTA and launch
   float2 *d_hp = nullptr;        // the training step's packed H
   float *d_loss_part = nullptr;  // per-CTA loss sums of the training step
   int fwd_grid = 0, bwd_grid = 0, step_grid = 0;
@@ -614,6 +614,24 @@ void filter_destroy(fft_plan_impl *pl) {
   }
   delete f;
   pl->filter = nullptr;
+}
+
+// The backward below 8192 points runs in launches of at most kSumRows rows per
+// row slot, each with its own rows of sums, so that no FP32 sum runs over more
+// than kSumRows rows in order however large the batch; the pairwise tree adds
+// them all.  (2^25 points are 18 rows per slot at most: one launch.)  From 8192
+// points on the one launch's CTAs, two per SM or one, add their rows in order.
+constexpr int kSumRows = 32;
+struct BwdLaunches {
+  int64_t rows;  // of each launch but the last
+  int64_t sums;  // rows of sums of all
+};
+static BwdLaunches bwd_launches(const FilterVariant &v, int N, int64_t batch, int grid) {
+  const int64_t round = (int64_t)grid * v.tb;
+  if (N >= 8192 || batch <= kSumRows * round) return {batch, grid};
+  const int64_t rows = kSumRows * round, full = (batch - 1) / rows;
+  const int64_t rest = (batch - full * rows + v.tb - 1) / v.tb;
+  return {rows, full * grid + std::min<int64_t>(grid, rest)};
 }
 
 // CTAs of kernel k that are resident on the GPU at once.  The occupancy query
@@ -698,7 +716,8 @@ fft_status_t fft_filter_plan(fft_plan_t *out, int N, int64_t batch) {
     f->step_grid = grid(v.step);
     if (f->fwd_grid < 1 || f->bwd_grid < 1 || f->step_grid < 1) return fail(FFT_ERR_CUDA);
     const int64_t row = (int64_t)sizeof(float2) * N;
-    pl->scratch_bytes = std::max(f->bwd_grid, f->step_grid) * row;
+    pl->scratch_bytes =
+        std::max<int64_t>(bwd_launches(v, N, batch, f->bwd_grid).sums, f->step_grid) * row;
     if (!alloc(&f->d_work, pl->scratch_bytes) || !alloc(&f->d_hp, row) ||
         !alloc(&f->d_loss_part, (int64_t)sizeof(float) * f->step_grid))
       return fail(FFT_ERR_ALLOC);
@@ -769,14 +788,22 @@ static fft_status_t filter_backward(fft_plan_t plan, const void *g_y, const void
   b.out = (float2 *)grad_x;
   b.partial = f->d_work;
   b.tw = pl->d_tw;
-  b.batch = pl->batch;
   b.inv_n = 1.0f / (float)N;
   const FilterKernel &k = natural ? f->v.bwd_natural : f->v.bwd;
-  void *args[] = {&b};
-  if ((s = cuda_status(launch_pdl(k.fn, dim3((unsigned)f->bwd_grid), dim3(f->v.threads),
-                                  f->v.smem, st, args))) != FFT_OK)
-    return s;
-  return grad_h_tree(f->d_work, (float2 *)grad_H, N, f->bwd_grid, st, f->v.shape, LossSum{});
+  const BwdLaunches l = bwd_launches(f->v, N, pl->batch, f->bwd_grid);
+  for (int64_t r0 = 0; r0 < pl->batch; r0 += l.rows) {
+    b.batch = std::min(l.rows, pl->batch - r0);
+    const int64_t grid = std::min<int64_t>(f->bwd_grid, (b.batch + f->v.tb - 1) / f->v.tb);
+    void *args[] = {&b};
+    if ((s = cuda_status(launch_pdl(k.fn, dim3((unsigned)grid), dim3(f->v.threads), f->v.smem, st,
+                                    args))) != FFT_OK)
+      return s;
+    b.in += b.batch * N;
+    b.x_save += b.batch * N;
+    b.out += b.batch * N;
+    b.partial += grid * N;
+  }
+  return grad_h_tree(f->d_work, (float2 *)grad_H, N, l.sums, st, f->v.shape, LossSum{});
 }
 
 fft_status_t fft_filter_forward(fft_plan_t plan, const void *x, const void *H, void *y,
