@@ -27,7 +27,10 @@
  * status word read by fft_last_device_status() after a synchronisation.
  *
  * Thread safety: a plan may be executed from one host thread at a time;
- * different plans are independent.
+ * different plans are independent.  Executions of one plan on several streams
+ * must not overlap on the GPU where the plan owns memory that they write, such
+ * as the four-step scratch, a ragged plan's counters and the sums behind a
+ * filter's grad_H and loss (its y and grad_x do not depend on them).
  */
 #ifndef FFTGB_H_
 #define FFTGB_H_

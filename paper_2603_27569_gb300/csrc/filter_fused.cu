@@ -405,7 +405,9 @@ filter_bwd_kernel(FilterArgs a) {
 // grad_x = F^H (conj(H) g_z).  X and g_y never leave the SM: a row reads x
 // and m and writes y and grad_x, 28 bytes per point.  Tensor memory holds the
 // sums and X, so H comes from a copy in packed order that a small kernel
-// before this one leaves in the plan (coalesced 16-byte loads).
+// before this one leaves in grad_H (coalesced 16-byte loads): the caller's
+// buffer, which nothing else uses before the tree writes the result there, so
+// that steps of one plan on two streams read each its own H.
 struct FilterStepArgs {
   const float2 *x;
   const float2 *hp;   // H, packed order
@@ -600,7 +602,7 @@ static bool filter_variant(int N, FilterVariant *v) {
 struct FilterState {
   FilterVariant v;
   float2 *d_work = nullptr;      // grad_H sums, one row per CTA and launch
-  float2 *d_hp = nullptr;        // the training step's packed H
+  float2 *d_hp = nullptr;        // the training step's packed H, where grad_H cannot hold it
   float *d_loss_part = nullptr;  // per-CTA loss sums of the training step
   int fwd_grid = 0, bwd_grid = 0, step_grid = 0;
 };
@@ -853,7 +855,12 @@ fft_status_t fft_filter_step(fft_plan_t plan, const void *x, const void *H, cons
   if (y && overlap(y, bytes, grad_x, bytes)) return FFT_ERR_INVALID_VALUE;
   FilterStepArgs a{};
   a.x = (const float2 *)x;
-  a.hp = f->d_hp;
+  // grad_H may share memory with an input, which must stay until it is read
+  const int64_t hb = (int64_t)sizeof(float2) * N;
+  const bool own = overlap(grad_H, hb, H, hb) || overlap(grad_H, hb, x, bytes) ||
+                   overlap(grad_H, hb, mask, bytes / 2);
+  float2 *hp = own ? f->d_hp : (float2 *)grad_H;
+  a.hp = hp;
   a.mask = mask;
   a.y = (float2 *)y;
   a.gx = (float2 *)grad_x;
@@ -864,7 +871,7 @@ fft_status_t fft_filter_step(fft_plan_t plan, const void *x, const void *H, cons
   a.inv_n = 1.0f / (float)N;
   const float2 *h = (const float2 *)H;
   int n = N;
-  void *pack[] = {&h, &f->d_hp, &n, &f->v.shape};
+  void *pack[] = {&h, &hp, &n, &f->v.shape};
   if ((s = cuda_status(launch_pdl((const void *)pack_h_kernel, dim3((N + 255) / 256), dim3(256), 0,
                                   st, pack))) != FFT_OK)
     return s;
