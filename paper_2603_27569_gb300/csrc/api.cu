@@ -371,11 +371,11 @@ static const KernelEntry *plain_column(int L, int64_t ncols, int64_t cols) {
   const KernelEntry *wide = default_column(L, 3);
   if (wide && ncols % wide->TB == 0) {
     int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-        cols / wide->TB >= sms)
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      cudaGetLastError();
+    else if (cols / wide->TB >= sms)
       return wide;
-    cudaGetLastError();
   }
   return default_column(L, 0);
 }
