@@ -165,7 +165,8 @@ def _raw(x: torch.Tensor, direction: int, precision: int, flags: int, out=None) 
     N = x.shape[-1]
     batch = x.numel() // N if N else 0
     plan = get_plan(N, batch, direction, precision, flags, x.device)
-    y = plan.exec(x.contiguous(), out)
+    # (the memory of a lazy conjugate holds the values unconjugated)
+    y = plan.exec(x.resolve_conj().contiguous(), out)
     return y if y.shape == x.shape else y.view(x.shape)
 
 
@@ -177,7 +178,7 @@ class _FFTFn(torch.autograd.Function):
 
     @staticmethod
     def backward(ctx, g):
-        gx = _raw(g.contiguous(), ctx.direction, ctx.precision, ctx.flags | B.FFT_FLAG_ADJOINT)
+        gx = _raw(g, ctx.direction, ctx.precision, ctx.flags | B.FFT_FLAG_ADJOINT)
         return gx, None, None, None
 
 
@@ -205,7 +206,7 @@ def fft_host(x: torch.Tensor, inverse: bool = False, device=None) -> torch.Tenso
     N = x.shape[-1]
     batch = x.numel() // N
     plan = get_plan(N, batch, B.FFT_INVERSE if inverse else B.FFT_FORWARD, 0, 0, device)
-    return plan.exec_host(x.contiguous()).view(x.shape)
+    return plan.exec_host(x.resolve_conj().contiguous()).view(x.shape)
 
 
 class ColumnPlan:
@@ -266,6 +267,7 @@ def fft_columns(x: torch.Tensor, inverse: bool = False) -> torch.Tensor:
     are); returns a tensor of the same shape and strides."""
     if x.dim() < 2 or x.stride(-1) != 1:
         raise ValueError("need [..., L, ncols] with a contiguous last dimension")
+    x = x.resolve_conj()
     lead = x.shape[:-2]
     if len(lead) > 1:
         x = x.reshape((-1,) + tuple(x.shape[-2:]))
@@ -297,7 +299,7 @@ class _SpectralFilterFn(torch.autograd.Function):
         N = x.shape[-1]
         batch = x.numel() // N
         xc = x.contiguous()
-        Hc = H.contiguous()
+        Hc = H.resolve_conj().contiguous()
         X = _raw(xc, B.FFT_FORWARD, 0, 0)                       # F x
         Z = torch.empty_like(X)
         st = torch.cuda.current_stream(x.device)
@@ -313,7 +315,7 @@ class _SpectralFilterFn(torch.autograd.Function):
         N = X.shape[-1]
         batch = X.numel() // N
         st = torch.cuda.current_stream(X.device)
-        gz = _raw(gy.contiguous(), B.FFT_INVERSE, 0, B.FFT_FLAG_ADJOINT)  # G^H g_y = F g_y / N
+        gz = _raw(gy, B.FFT_INVERSE, 0, B.FFT_FLAG_ADJOINT)  # G^H g_y = F g_y / N
         grad_x = grad_H = None
         if ctx.needs_input_grad[1]:
             grad_H = torch.empty(N, dtype=torch.complex64, device=X.device)
@@ -387,8 +389,8 @@ class _FusedSpectralFilterFn(torch.autograd.Function):
     def forward(ctx, x, H):
         N = x.shape[-1]
         batch = x.numel() // N
-        xc = x.contiguous()
-        Hc = H.contiguous()
+        xc = x.resolve_conj().contiguous()
+        Hc = H.resolve_conj().contiguous()
         plan = _filter_plan(N, batch, x.device)
         y = torch.empty_like(xc)
         need_grad = ctx.needs_input_grad[0] or ctx.needs_input_grad[1]
@@ -403,7 +405,7 @@ class _FusedSpectralFilterFn(torch.autograd.Function):
         X, H = ctx.saved_tensors
         gx = torch.empty_like(X)
         gH = X.new_empty(ctx.shape[-1])
-        B.fft_filter_backward_packed(ctx.plan.handle, gy.contiguous(), H, X, gx, gH,
+        B.fft_filter_backward_packed(ctx.plan.handle, gy.resolve_conj().contiguous(), H, X, gx, gH,
                                      _raw_stream(X.get_device()))
         if gx.shape != ctx.shape:
             gx = gx.view(ctx.shape)
@@ -441,11 +443,11 @@ def spectral_filter_step(x: torch.Tensor, H: torch.Tensor, mask: torch.Tensor,
     _check_filter(x, H)
     N = x.shape[-1]
     batch = x.numel() // N
-    xc = x.contiguous()
-    Hc = H.detach().contiguous()
+    xc = x.resolve_conj().contiguous()
+    Hc = H.detach().resolve_conj().contiguous()
     if mask.device != x.device:
         raise ValueError(f"mask must live on {x.device}, not {mask.device}")
-    m = (mask if mask.dtype == torch.float32 else mask.to(torch.float32)).contiguous()
+    m = (mask if mask.dtype == torch.float32 else mask.to(torch.float32)).resolve_neg().contiguous()
     if m.shape != x.shape:
         raise ValueError("mask must have x's shape")
     plan = _filter_plan(N, batch, x.device)
