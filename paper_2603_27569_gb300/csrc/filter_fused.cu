@@ -255,8 +255,13 @@ struct FilterArgs {
   float inv_n;
 };
 
-// NATURAL: the saved spectrum leaves in natural order, staged through the row
-// buffer (an exchange and three row barriers more than the packed order).
+// NATURAL: the saved spectrum leaves in natural order.  With two butterflies
+// per thread (8192) registers m and m + P / 2 are adjacent frequencies and two
+// lanes fill a sector, so the pairs are stored as they are.  The other lengths
+// hold single points there and stage through the row buffer (an exchange and
+// three row barriers more than the packed order).  Staged / stored directly,
+// one row and 2^25 points, us: 8192 9.2 / 8.7 and 169 / 161; 4096 5.4 / 5.7 and
+// 161 / 185; 16384 16.5 / 17.3 and 195 / 210.
 template <class R, int TB, bool NATURAL>
 __global__ void __launch_bounds__(TB *R::T, filter_min_ctas<R, TB>(FK_FWD))
 filter_fwd_kernel(FilterArgs a) {
@@ -287,7 +292,13 @@ filter_fwd_kernel(FilterArgs a) {
     r.template forward<TB>(v, cta.tw);
     if (a.x_save) {
       float2 *xs = a.x_save + (active ? row : 0) * N;
-      if constexpr (NATURAL) {
+      if constexpr (NATURAL && R::QB == 2) {
+        if (active) {
+#pragma unroll
+          for (int m = 0; m < P / 2; ++m)
+            __stcs(reinterpret_cast<float4 *>(xs + r.freq(m)), pack2(v[m], v[m + P / 2]));
+        }
+      } else if constexpr (NATURAL) {
         R::template row_sync<TB>(cta.b);  // every sub-row has been read
 #pragma unroll
         for (int m = 0; m < P; ++m) cta.buf[cta.at(r.freq(m))] = v[m];
