@@ -84,6 +84,20 @@ __host__ __device__ constexpr int filter_min_ctas(FilterKind k) {
   return 65536 / (TB * R::T * regs);
 }
 
+// Does the tensor-memory allocation stand before the first row's loads, or
+// behind them, covered by their latency but with the row's registers held
+// across it?  Measured, 2^25 points (1500 rows), us, before / behind: forward
+// 256 93.3 / 93.1, 1024 101.2 / 102.4 (8.4 / 8.6), 8192 134.0 / 135.7, 16384
+// 152.0 / 152.7; backward 256 150 / 141, 512 145.5 / 142.4 (11.1 / 11.4), 1024
+// 141.5 / 142.2 (14.9 / 16.4), 2048 149.1 / 147.3 (23.0 / 22.3), 4096 166 / 167,
+// 8192 175 / 177; step 1024 221 / 232, 2048 241 / 251, 4096 286 / 277, 8192 equal.
+template <class R>
+__host__ __device__ constexpr bool allocate_first(FilterKind k) {
+  return k == FK_FWD   ? R::N >= 1024
+         : k == FK_BWD ? R::N == 1024 || R::N >= 4096
+                       : R::N <= 2048;
+}
+
 // What the filter kernels share: the CTA's tables and tensor memory, this
 // thread's row slot, and the loads of its points.
 template <class R, int TB, int NARRAYS>
@@ -108,11 +122,7 @@ struct FilterCta {
     R::Rows::copy(tw, tables, tid, NT);
   }
   // After the wait (tmem.cuh): warp 0 allocates, and the barrier publishes the
-  // address and the tables.  The allocation stands behind the first row's
-  // loads, whose latency covers it, except in the step of several rows per
-  // CTA, where the row held across it cost registers (2^25 points, us, before
-  // / behind the loads: step 1024 221 / 232, 2048 241 / 251, 4096 286 / 277;
-  // backward 256 153 / 140, 4096 175 / 168, 8192 179 / 177).
+  // address and the tables (and H, where it is staged).
   __device__ __forceinline__ uint32_t *slot() const { return reinterpret_cast<uint32_t *>(tw + R::TW); }
   __device__ __forceinline__ void allocate() const {
     if (warp == 0) tmem_alloc_warp(slot(), NCOL);
@@ -176,12 +186,11 @@ struct FilterCta {
       }
     }
   }
+  __device__ __forceinline__ void land_h() const {  // publish() follows
+    if constexpr (STAGE_H) asm volatile("cp.async.wait_all;" ::: "memory");
+  }
   __device__ __forceinline__ void stash_h(const R &r, const float2 *H, bool conj, uint32_t t) const {
     constexpr int C = kChunk<P>;
-    if constexpr (STAGE_H) {
-      asm volatile("cp.async.wait_all;" ::: "memory");
-      R::template row_sync<TB>(b);
-    }
 #pragma unroll
     for (int c = 0; c < P / C; ++c) {
       float h[2 * C];
@@ -273,6 +282,7 @@ filter_fwd_kernel(FilterArgs a) {
   const int lt = cta.lt;
   const long long ntiles = (a.batch + TB - 1) / TB;
   long long tile = blockIdx.x;
+  if constexpr (allocate_first<R>(FK_FWD)) cta.allocate();
   cta.fetch_h(a.H);
   float2 v[P];
   {
@@ -280,7 +290,8 @@ filter_fwd_kernel(FilterArgs a) {
     const bool on = row < a.batch;
     cta.load(v, a.in + (on ? row : 0) * N, lt, on);
   }
-  cta.allocate();
+  if constexpr (!allocate_first<R>(FK_FWD)) cta.allocate();
+  cta.land_h();
   cta.publish();
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   cta.stash_h(r, a.H, a.conj_h, cta.array(0));
@@ -339,6 +350,7 @@ filter_bwd_kernel(FilterArgs a) {
   const int lt = cta.lt;
   const long long ntiles = (a.batch + TB - 1) / TB;
   long long tile = blockIdx.x;
+  if constexpr (allocate_first<R>(FK_BWD)) cta.allocate();
   cta.fetch_h(a.H);
   float2 v[P];
   {
@@ -347,7 +359,8 @@ filter_bwd_kernel(FilterArgs a) {
     cta.load(v, a.in + (on ? row : 0) * N, lt, on);
   }
   cta.prefetch(a.x_save, tile, a.batch, sizeof(float2));
-  cta.allocate();
+  if constexpr (!allocate_first<R>(FK_BWD)) cta.allocate();
+  cta.land_h();
   cta.publish();
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const uint32_t t_sum = cta.array(0), t_h = cta.array(1);
@@ -447,7 +460,7 @@ filter_step_kernel(FilterStepArgs a) {
   extern __shared__ __align__(128) float2 smem[];
   FilterCta<R, TB, 2> cta(smem, a.tw);
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if constexpr (TB > 1) cta.allocate();
+  if constexpr (allocate_first<R>(FK_STEP)) cta.allocate();
   const R r(cta.buf, cta.lt, cta.b);
   const int lt = cta.lt;
   const long long ntiles = (a.batch + TB - 1) / TB;
@@ -458,7 +471,7 @@ filter_step_kernel(FilterStepArgs a) {
     const bool on = row < a.batch;
     cta.load(v, a.x + (on ? row : 0) * N, lt, on);
   }
-  if constexpr (TB == 1) cta.allocate();
+  if constexpr (!allocate_first<R>(FK_STEP)) cta.allocate();
   cta.publish();
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const uint32_t t_sum = cta.array(0), t_x = cta.array(1);
