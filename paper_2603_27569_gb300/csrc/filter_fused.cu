@@ -28,13 +28,13 @@
 // order (five exchanges per pair, generic accesses, twiddle rows through L1;
 // three kernels for the backward below 8192) / now:
 //            forward     + spectrum   backward     step
-//     256    134 / 93    155 / 134    293 / 144    367 / 196
-//    1024    174 / 102   196 / 136    288 / 143    481 / 219
-//    4096    177 / 131   191 / 139    295 / 169    457 / 278
-//    8192    162 / 134   181 / 146    212 / 176    359 / 296
-//   16384    204 / 153   226 / 164    258 / 210    425 / 337
+//     256    134 / 91    155 / 131    293 / 140    367 / 182
+//    1024    174 / 101   196 / 133    288 / 141    481 / 221
+//    4096    177 / 131   191 / 140    295 / 166    457 / 277
+//    8192    162 / 134   181 / 146    212 / 175    359 / 297
+//   16384    204 / 152   226 / 163    258 / 206    425 / 340
 // (spectrum and backward in packed order; in natural order, for callers of
-// the unpacked entry points, 130..190 and 146..245.)
+// the unpacked entry points, 130..193 and 146..244.)
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -70,17 +70,17 @@ __host__ __device__ constexpr size_t filter_smem() {
   return sizeof(float2) * ((size_t)TB * R::BUF + R::TW + 2);
 }
 // CTAs per SM that registers are budgeted for: 128 per thread with 32 points;
-// with 16 points 80 (three CTAs of 256 threads, no spills) or 64 (four, some
-// words spilled), whichever measured faster per kernel (2^25 points, 80 / 64
-// registers: 1024 forward 102 / 106, backward 146 / 158, step 231 / 254 us;
-// 4096 131 / 137, 177 / 171, 297 / 290; 256 93 / 93, 144 / 161, 226 / 207).
+// with 16 points 80 (three CTAs of 256 threads) or 64 (four), whichever measured
+// faster (2^25 points, us, 80 / 64 registers, at 256, 512, 1024, 2048, 4096:
+// forward 93 / 94, 96 / 110, 102 / 102, 112 / 109, 131 / 135; backward 141 /
+// 157, 142 / 179, 142 / 170, 147 / 179, 169 / 168; step 182 / 198, 215 / 237,
+// 221 / 248, 241 / 258, 293 / 277).  Spills by -Xptxas -v, bytes: forward none;
+// backward 0 to 32 at 80 registers, 72 to 84 at 64, 40 to 48 at 128; step 0 to
+// 36, 28, 120 to 152.
 enum FilterKind { FK_FWD, FK_BWD, FK_STEP };
 template <class R, int TB>
 __host__ __device__ constexpr int filter_min_ctas(FilterKind k) {
-  const int regs = R::P == 32                      ? 128
-                   : (R::N == 4096 && k != FK_FWD) ? 64
-                   : (R::N == 256 && k == FK_STEP) ? 64
-                                                   : 80;
+  const int regs = R::P == 32 ? 128 : R::N == 4096 && k != FK_FWD ? 64 : 80;
   return 65536 / (TB * R::T * regs);
 }
 
@@ -90,11 +90,12 @@ __host__ __device__ constexpr int filter_min_ctas(FilterKind k) {
 // 256 93.3 / 93.1, 1024 101.2 / 102.4 (8.4 / 8.6), 8192 134.0 / 135.7, 16384
 // 152.0 / 152.7; backward 256 150 / 141, 512 145.5 / 142.4 (11.1 / 11.4), 1024
 // 141.5 / 142.2 (14.9 / 16.4), 2048 149.1 / 147.3 (23.0 / 22.3), 4096 166 / 167,
-// 8192 175 / 177; step 1024 221 / 232, 2048 241 / 251, 4096 286 / 277, 8192 equal.
+// 8192 175 / 176, 16384 210 / 206; step 1024 221 / 232, 2048 241 / 251, 4096
+// 286 / 277, 8192 equal.
 template <class R>
 __host__ __device__ constexpr bool allocate_first(FilterKind k) {
   return k == FK_FWD   ? R::N >= 1024
-         : k == FK_BWD ? R::N == 1024 || R::N >= 4096
+         : k == FK_BWD ? R::N == 1024 || R::N == 4096 || R::N == 8192
                        : R::N <= 2048;
 }
 
