@@ -224,10 +224,13 @@ fft_status_t fft_plan_config(fft_plan_t *out, int N, int64_t batch, int directio
  * aligned; in == out is allowed, partial overlap is FFT_ERR_INVALID_VALUE.
  * For a ragged plan, in and out are the packed base pointers the plan's
  * offsets index.  stream: cudaStream_t or NULL.  Asynchronous.
- * Stream order holds as for any launch: the single-CTA, filter and
- * (up to 2048-point) column kernels use programmatic dependent launch, so
- * their CTAs may become resident while the previous kernel of the stream
- * finishes, but they read and write nothing before it has completed.
+ * Stream order holds as for any launch: the single-CTA kernels (FP32, 16-bit
+ * storage, 32768 halves), the column, tensor-core and filter kernels and the
+ * grad_H sum use programmatic dependent launch, so their CTAs may become
+ * resident while the previous kernel of the stream finishes.  Before it has
+ * completed they touch none of the caller's buffers and no memory that kernels
+ * write, and hold no tensor memory; the filter kernels read their twiddle
+ * tables, which are constant from the plan's creation on.
  * Paper: Sec. II-A (fft_exec(plan, in, out, stream) over the DFT defined
  * there); Sec. II-B (Stockham autosort: natural-order output).
  */

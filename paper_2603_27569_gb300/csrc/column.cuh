@@ -68,8 +68,8 @@ struct ColumnLoopArgs : ColumnArgs {
   unsigned ntiles;  // tiles of the launch
 };
 
-// Row pitch of the tile whose last exchange is read transposed: 16 consecutive
-// lanes read outputs lt of one column at distinct bank pairs.
+// Row pitch of a tile that is read transposed, in its last exchange or staged:
+// 16 consecutive lanes read outputs lt of one column at distinct bank pairs.
 template <int C>
 __host__ __device__ constexpr int transposed_pitch() {
   return C + 1;
@@ -198,8 +198,8 @@ column_kernel(ColumnArgs args) {
     }
   }
   if constexpr (TRANSPOSED) {
-    // out[col * L + k]: stage through a tile padded to C + 1 columns.
-    constexpr int LD = C + 1;
+    // out[col * L + k]: stage through a padded tile.
+    constexpr int LD = transposed_pitch<C>();
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < P; ++m) smem[final_index<L, P, SC>(lt, m) * LD + c] = a[m];

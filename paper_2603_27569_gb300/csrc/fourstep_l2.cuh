@@ -170,10 +170,10 @@ fourstep_l2_kernel(FourstepL2Args a) {
             float2 *dst = slot + (long long)(c0 + c2) * L + lt2;
 #pragma unroll
             for (int m = 0; m < P; ++m) __stcg(dst + m * T, v[m]);
-          } else {  // through a tile padded to C + 1 columns
+          } else {  // through a padded tile
             run_passes<L, P, D, SC, 0>(v, ltp, bufp, twp, Interleaved<C>{cp});
             phase1_twiddle_staged<P, D>(v, ltp, c0 + cp, L, a.tw_a, a.tw_b);
-            constexpr int LD = C + 1;
+            constexpr int LD = transposed_pitch<C>();
             __syncthreads();
 #pragma unroll
             for (int m = 0; m < P; ++m) smem[final_index<L, P, SC>(lt, m) * LD + c] = v[m];

@@ -121,7 +121,7 @@ inline KernelEntry column_entry() {
   e.P = P;
   e.TB = C;
   e.threads = C * (L / P);
-  e.smem = sizeof(float2) * (size_t)L * (VAR ? transposed_pitch<C>() : C);  // or C + 1, staged
+  e.smem = sizeof(float2) * (size_t)L * (VAR ? transposed_pitch<C>() : C);
   e.tw_by_column = VAR && merged_transpose<L, P, SC>();
   fill_radix<SC>(e);
   e.is_default = DEF;

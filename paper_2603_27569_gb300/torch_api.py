@@ -445,8 +445,8 @@ def spectral_filter_step(x: torch.Tensor, H: torch.Tensor, mask: torch.Tensor,
                          keep_y: bool = True):
     """One fused training step of the filter under L = sum(mask * |y|^2):
     returns (y or None, L, grad_x, grad_H) from one persistent kernel per call
-    (C ABI: fft_filter_step; N = 8192 or 16384, x [..., N] complex64, mask the
-    same shape as float32)."""
+    (C ABI: fft_filter_step; N = 256..16384, x [..., N] and H [N] complex64,
+    mask of x's shape as float32; grad_H is [N])."""
     _check_filter(x, H)
     N = x.shape[-1]
     batch = x.numel() // N
