@@ -37,3 +37,26 @@ def test_grad_h_in_an_input(N, rows, where):
 
     for a, b in zip(run(None), run(where)):
         assert np.array_equal(a.view(np.uint32), b.view(np.uint32))
+
+
+@pytest.mark.parametrize("N,rows", [(1024, 6001), (16384, 160)])
+def test_one_grad_h_buffer_for_calls_back_to_back(N, rows):
+    # the buffer holds each call's packed H, then its result, with no host
+    # synchronisation in between
+    x, m = to_dev(synth.gaussian((rows, N), seed=1)), to_dev(synth.real_mask((rows, N), seed=3))
+    Hs = [to_dev(synth.gaussian(N, seed=10 + i)) for i in range(6)]
+    loss = torch.empty((), device="cuda")
+    st = torch.cuda.current_stream()
+    plan = fg.fft_filter_plan(N, rows)
+    gH = torch.empty_like(Hs[0])
+    got = []
+    for H in Hs:
+        y, gx = torch.empty_like(x), torch.empty_like(x)
+        fg.fft_filter_step(plan, x, H, m, y, gx, gH, loss, st)
+        got.append((y, gx, gH.clone()))
+    fg.fft_destroy(plan)
+    for H, outs in zip(Hs, got):
+        torch.cuda.synchronize()
+        want = fg.spectral_filter_step(x, H, m)
+        for a, b in zip(outs, (want[0], want[2], want[3])):
+            assert np.array_equal(to_host(a).view(np.uint32), to_host(b).view(np.uint32))
