@@ -89,6 +89,14 @@ __device__ __forceinline__ L2Item l2_item(long long w, long long TT, int lag) {
 }
 
 // Register budget 64 per thread (65536 / 64 threads' worth of CTAs per SM).
+//
+// The pass twiddles are read from a shared-memory copy made once per CTA.  The
+// acquire loads of the counters empty L1 at every item, so through L1 all CTAs
+// fetched the same few lines from L2 again and again, and the time depended on
+// which L2 slices those lines fell into, that is, on what else was allocated:
+// 2^25 points at 16384, chunks of 8 rows, between 161 and 191 us as other plans
+// came and went; now 160 to 162, and 4096 162 to 172 (182 to 192), 65536 157
+// (159).
 template <int L, int P, int C, int D, class SC>
 __global__ void __launch_bounds__(C *(L / P), 1024 / (C * (L / P)))
 fourstep_l2_kernel(FourstepL2Args a) {
@@ -110,6 +118,8 @@ fourstep_l2_kernel(FourstepL2Args a) {
   // while the current one is processed (a CTA holding item w and the next
   // claimed item still only ever waits on items below w).
   if (threadIdx.x == 0) s_item[0] = (long long)atomicAdd(a.counters, 1u);
+  float2 *tws = smem + L * transposed_pitch<C>();
+  for (int i = threadIdx.x; i < SC::tw_total(); i += NT) tws[i] = __ldg(a.tw + i);
   __syncthreads();
   int cur = 0;
   while (true) {
@@ -149,16 +159,10 @@ fourstep_l2_kernel(FourstepL2Args a) {
         }
         // Opaque per item: keeps table addresses and loads inside the loop, the
         // buffer through an offset so that it stays visibly shared memory.
-        // Columns of 64 points, two warps per CTA, measured faster with the
-        // pointer itself opaque (N = 4096, 2^25 points, chunks of 8 / 16 rows:
-        // 180 / 198 us, with the offset 191 / 204; 16384 166 and 159, 65536
-        // with chunks of 16 rows 161 and 156, so they take the offset).
         const float2 *twp = a.tw;
-        float2 *bufp = smem;
         int ltp = lt, cp = c, zero = 0;
         asm volatile("" : "+l"(twp), "+r"(ltp), "+r"(cp), "+r"(zero));
-        if constexpr (L < 128) asm volatile("" : "+l"(bufp));
-        else bufp = smem + zero;
+        float2 *bufp = smem + zero;
         if (it.p1) {
           // A[n1][k2] at slot + n1 * L + k2
           if constexpr (merged_transpose<L, P, SC>()) {  // the last exchange read transposed (column.cuh)
@@ -171,7 +175,7 @@ fourstep_l2_kernel(FourstepL2Args a) {
 #pragma unroll
             for (int m = 0; m < P; ++m) __stcg(dst + m * T, v[m]);
           } else {  // through a padded tile
-            run_passes<L, P, D, SC, 0>(v, ltp, bufp, twp, Interleaved<C>{cp});
+            run_passes_shared<L, P, C, D, SC, 0>(v, ltp, cp, bufp, tws + zero);
             phase1_twiddle_staged<P, D>(v, ltp, c0 + cp, L, a.tw_a, a.tw_b);
             constexpr int LD = transposed_pitch<C>();
             __syncthreads();
@@ -187,7 +191,7 @@ fourstep_l2_kernel(FourstepL2Args a) {
             }
           }
         } else {
-          run_passes<L, P, D, SC, 0>(v, ltp, bufp, twp, Interleaved<C>{cp});
+          run_passes_shared<L, P, C, D, SC, 0>(v, ltp, cp, bufp, tws + zero);
           // consumed: drop this tile's L row segments (C points = 128 bytes) from L2
           __syncthreads();
           for (int q = threadIdx.x; q < L; q += NT)

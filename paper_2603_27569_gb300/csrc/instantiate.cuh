@@ -139,7 +139,7 @@ inline KernelEntry fourstep_l2_entry() {
   e.P = P;
   e.TB = C;
   e.threads = C * (L / P);
-  e.smem = sizeof(float2) * (size_t)L * (C + 1);
+  e.smem = sizeof(float2) * ((size_t)L * transposed_pitch<C>() + SC::tw_total());
   e.tw_by_column = merged_transpose<L, P, SC>();
   fill_radix<SC>(e);
   e.is_default = 0;
